@@ -17,9 +17,11 @@
 // update and theta^+ for a right-to-left one.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstddef>
 #include <mutex>
+#include <vector>
 
 #include "common.cuh"
 
@@ -204,6 +206,64 @@ __global__ void __launch_bounds__(128) jacobi_kernel(typename cplx<R>::T* __rest
   }
 }
 
+// Rotation of a pair (u, v) with alpha = |u|^2, beta = |v|^2, gamma = u^+ v:
+//   u' = c (u - conj(sigma) v),  v' = c (v + sigma u),  c = 1 / sqrt(1 + |sigma|^2),
+//   sigma = -sgn(delta) 2 gamma / (|delta| + sqrt(delta^2 + 4 |gamma|^2)),  delta = alpha - beta
+// zeroes gamma (the smaller angle).  Any sigma gives a unitary map as long as
+// c belongs to it, so sigma itself may carry a relative rounding error; no
+// phase has to be normalised.  One square root, one reciprocal square root and
+// two quotients in all (the form with a separate phase took four and seven,
+// about half of the instructions of a short pair).
+// false: the pair is skipped (a numerically zero column, or |gamma| <= tol
+// sqrt(alpha beta)); rel2 = |gamma|^2 / (alpha beta).
+// mst = c - 1 = -|sigma|^2 c^2 / (1 + c), accurate when c rounds to 1 (the plain
+// form would grow every rotated column by |sigma|^2 / 2).
+__device__ __forceinline__ bool jacobi_params(float al, float be, float gr, float gi, float tiny, float tol, float2& cs,
+                                              float& mst, float& rel2) {
+  const float g2 = gr * gr + gi * gi, ab = al * be;
+  if (!(al > tiny) || !(be > tiny) || !(g2 > tol * tol * ab)) return false;
+  rel2 = __fdividef(g2, fminf(ab, 8e37f));   // __fdividef returns 0 for divisors beyond 2^126
+  const float de = al - be;
+  const float h = fabsf(de) + sqrtf(fmaf(de, de, 4.f * g2));
+  const float k = (de >= 0.f ? -2.f : 2.f) / h;
+  const float sr = k * gr, si = k * gi;
+  const float q = sr * sr + si * si;
+  const float c0 = rsqrtf(1.f + q);
+  mst = -__fdividef(q * c0 * c0, 1.f + c0);
+  const float c = 1.f + mst;
+  cs = make_float2(c * sr, c * si);
+  return true;
+}
+
+// FP64: the same rotation (c instead of c - 1).  GB300 issues an FP64
+// instruction of a warp over 64 cycles of a quarter of its SM, so sigma comes
+// from FP32 arithmetic on values scaled by 2^-e, e the exponent of gamma (a
+// relative error of 1e-7 in sigma leaves 1e-7 of gamma, and the stopping rule
+// looks at the gammas themselves), and only what makes the map unitary is FP64:
+// with c0 = rsqrt(1 + |sigma|^2) rounded to FP32 and d = c0^2 (1 + |sigma|^2) - 1
+// ~ 1e-7, c = c0 (1 - d/2 + 3 d^2 / 8) is off by d^3.
+__device__ __forceinline__ bool jacobi_params(double al, double be, double gr, double gi, double tiny, double tol,
+                                              double2& cs, double& c, float& rel2) {
+  const double mg = fmax(fabs(gr), fabs(gi));
+  if (!(al > tiny) || !(be > tiny) || !(mg > 0)) return false;
+  const double isg = __hiloint2double(0x7fe00000 - (__double2hiint(mg) & 0x7ff00000), 0);   // 2^-e
+  const float fr = (float)(gr * isg), fi = (float)(gi * isg);
+  const float g2 = fr * fr + fi * fi;                       // in [1, 8)
+  const float ab = (float)(al * isg) * (float)(be * isg);   // inf only below any tol
+  if (!(g2 > (float)(tol * tol) * ab)) return false;
+  rel2 = __fdividef(g2, fminf(ab, 8e37f));
+  const float de = (float)((al - be) * isg), ad = fabsf(de);
+  const float h = ad + (ad > 1e15f ? ad : sqrtf(fmaf(de, de, 4.f * g2)));
+  const float k = (de >= 0.f ? -2.f : 2.f) / h;
+  const double sr = (double)(k * fr), si = (double)(k * fi);
+  const double q = fma(sr, sr, si * si);
+  const double c0 = (double)rsqrtf(1.f + (float)q), c2 = c0 * c0;
+  const double d = fma(q, c2, c2 - 1.0);
+  c = fma(c0 * d, fma(d, 0.375, -0.5), c0);
+  cs = make_double2(c * sr, c * si);
+  return true;
+}
+
 // Register-resident variant for m <= 128*E: one CTA (128 threads) per column
 // pair, each thread holding E elements of both columns, so a pair costs one
 // load, one block reduction and one store.  Same rotation and stopping rule.
@@ -252,30 +312,26 @@ __global__ void __launch_bounds__(128) jacobi_reg_kernel(typename cplx<R>::T* __
         gr = red[buf][0][2] + red[buf][1][2] + red[buf][2][2] + red[buf][3][2];
         gi = red[buf][0][3] + red[buf][1][3] + red[buf][2][3] + red[buf][3][3];
         buf ^= 1;   // the next pair reduces into the other buffer: no second barrier
-        const R gabs = sqrt(gr * gr + gi * gi);
-        if (al <= tiny || be <= tiny || gabs <= tiny) continue;
-        const R rel = gabs / sqrt(al * be);
-        if (!(rel > tol)) continue;
-        local_off = fmaxf(local_off, (float)rel);
+        C2 cs;
+        R cm;      // FP64: c; complex64: c - 1
+        float rel2;
+        if (!jacobi_params(al, be, gr, gi, tiny, tol, cs, cm, rel2)) continue;
+        local_off = fmaxf(local_off, rel2);
         if (tid == 0) ++rot;
-        const R er = gr / gabs, ei = -gi / gabs;
-        const R zeta = (al - be) / (2 * gabs);
-        const R sg = zeta >= 0 ? R(1) : R(-1);
-        const R t = -sg / (fabs(zeta) + sqrt(R(1) + zeta * zeta));
-        const R c = R(1) / sqrt(R(1) + t * t);
-        const R sn = c * t;
-        const R mst = -sn * (sn / (R(1) + c));   // c - 1, accurate when c rounds to 1
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           const int i = tid + e * 128;
           if (i < m) {
-            const C2 ye{y[e].x * er - y[e].y * ei, y[e].x * ei + y[e].y * er};
-            u[i] = C2{x[e].x + (mst * x[e].x - sn * ye.x), x[e].y + (mst * x[e].y - sn * ye.y)};
-            v[i] = C2{ye.x + (sn * x[e].x + mst * ye.x), ye.y + (sn * x[e].y + mst * ye.y)};
+            // u' = c u - conj(c sigma) v,  v' = c v + c sigma u
+            C2 du{cm * x[e].x - (cs.x * y[e].x + cs.y * y[e].y), cm * x[e].y - (cs.x * y[e].y - cs.y * y[e].x)};
+            C2 dv{cm * y[e].x + (cs.x * x[e].x - cs.y * x[e].y), cm * y[e].y + (cs.x * x[e].y + cs.y * x[e].x)};
+            if constexpr (sizeof(R) == 4) { du.x += x[e].x; du.y += x[e].y; dv.x += y[e].x; dv.y += y[e].y; }
+            u[i] = du;
+            v[i] = dv;
           }
         }
       }
-      if (tid == 0 && local_off > 0.f) atomicMax(&ctl->off_bits[sweep & 1], __float_as_uint(local_off));
+      if (tid == 0 && local_off > 0.f) atomicMax(&ctl->off_bits[sweep & 1], __float_as_uint(sqrtf(local_off)));
       local_off = 0.f;
       if (!grid_barrier(ctl, nb)) {
         if (tid == 0 && rot) atomicAdd(&ctl->rotations, rot);
@@ -333,7 +389,7 @@ __device__ __forceinline__ void warp_sum4(float& a, float& b, float& c, float& d
 
 template <bool FIRST, int E>
 __device__ __forceinline__ void wp4_pair(float2 (&x)[E], const float2 (&y)[E], bool ok, float tiny, float tol,
-                                         float& local_off, unsigned long long& rot) {
+                                         float& local_off, unsigned& rot) {
   // (u, v) = (first, second) column: the same arithmetic in both warps of the
   // pair.  Packed FP32x2 FMAs: nu = (sum ux^2, sum uy^2), nv likewise,
   // p1 = (sum ux vx, sum uy vy), p2 = (sum ux vy, sum uy vx).
@@ -349,53 +405,28 @@ __device__ __forceinline__ void wp4_pair(float2 (&x)[E], const float2 (&y)[E], b
   }
   float al = nu.x + nu.y, be = nv.x + nv.y, gr = p1.x + p1.y, gi = p2.x - p2.y;
   warp_sum4(al, be, gr, gi);
-  const float gabs = sqrtf(gr * gr + gi * gi);
-  if (!ok || !(al > tiny) || !(be > tiny) || !(gabs > tiny)) return;
-  const float rel = gabs / sqrtf(al * be);
-  if (!(rel > tol)) return;
+  float2 cs;
+  float mst, rel2;
+  if (!ok || !jacobi_params(al, be, gr, gi, tiny, tol, cs, mst, rel2)) return;
   if (FIRST) {
-    local_off = fmaxf(local_off, rel);
-    if ((threadIdx.x & 31) == 0) ++rot;
+    local_off = fmaxf(local_off, rel2);
+    ++rot;
   }
-  const float er = gr / gabs, ei = -gi / gabs;
-  const float zeta = (al - be) / (2.f * gabs);
-  const float sg = zeta >= 0.f ? 1.f : -1.f;
-  const float t = -sg / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
-  const float c = 1.f / sqrtf(1.f + t * t);
-  const float sn = c * t;
-  // first: u' = c u - s e^{-i phi} v;  second: v' = s u + c e^{-i phi} v,
-  // applied as corrections of the column itself with tau = s / (1 + c), since
-  // c = 1 - s tau:  u' = u + (-s tau u - s e v),  v' = e v + (-s tau e v + s u)
-  // (e = e^{-i phi}).  For small rotations c rounds to 1 while c^2 + s^2 = 1 + t^2
-  // does not; the plain form then grows every column by t^2 / 2 per rotation,
-  // a bias that thousands of late-sweep rotations turn into ~1e-4 of s_1.
-  const float mst = -sn * (sn / (1.f + c));
+  // applied as corrections of the column itself: x + (mst x -+ c sigma y)
   const float2 MST{mst, mst};
-  if (FIRST) {
-    const float br = -sn * er, bi = -sn * ei;
-    const float2 BR{br, br}, BI{-bi, bi};
+  const float br = FIRST ? -cs.x : cs.x;
+  const float2 BR{br, br}, BI{-cs.y, cs.y};   // first: -conj(c sigma) v, second: c sigma u
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const float2 u = x[e], v = y[e];
-      const float2 d = __ffma2_rn(MST, u, __ffma2_rn(BR, v, __fmul2_rn(BI, make_float2(v.y, v.x))));
-      x[e] = make_float2(u.x + d.x, u.y + d.y);
-    }
-  } else {
-    const float2 ER{er, er}, EI{-ei, ei}, SN{sn, sn};
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const float2 u = y[e], v = x[e];
-      const float2 ev = __ffma2_rn(ER, v, __fmul2_rn(EI, make_float2(v.y, v.x)));
-      const float2 d = __ffma2_rn(MST, ev, __fmul2_rn(SN, u));
-      x[e] = make_float2(ev.x + d.x, ev.y + d.y);
-    }
+  for (int e = 0; e < E; ++e) {
+    const float2 d = __ffma2_rn(MST, x[e], __ffma2_rn(BR, y[e], __fmul2_rn(BI, make_float2(y[e].y, y[e].x))));
+    x[e] = make_float2(x[e].x + d.x, x[e].y + d.y);
   }
 }
 
 template <int SUB, int E, int VEC>
 __device__ __forceinline__ void wp4_subround(float2 (&x)[E], bool valid_me, const bool* valid_all, float2* sbuf,
                                              int m, int& buf, float tiny, float tol, float& local_off,
-                                             unsigned long long& rot) {
+                                             unsigned& rot) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int p = wp4_partner<SUB>(w);
   // columns are padded to 32 E rows in shared memory (rows >= m hold zeros in
@@ -450,7 +481,7 @@ __global__ void __launch_bounds__(256, 1) jacobi_wp4_kernel(float2* __restrict__
   const float conv = fmaxf(tol, 2e-3f);
   unsigned* done = block_rounds(ctl);      // rounds completed per column block
   int sweep = 0, buf = 0;
-  unsigned long long rot = 0;
+  unsigned rot = 0;
   for (; sweep < max_sweeps; ++sweep) {
     // slot of the sweep after next: every CTA read it at the end of sweep - 2,
     // before passing the barrier that ended sweep - 1
@@ -464,7 +495,7 @@ __global__ void __launch_bounds__(256, 1) jacobi_wp4_kernel(float2* __restrict__
         // the two blocks must have finished the previous round (point-to-point
         // instead of a grid barrier: no CTA waits for the slowest one)
         if (!wait_rounds(ctl, done, I, J, need)) {
-          if (lane == 0 && rot) atomicAdd(&ctl->rotations, rot);
+          if (lane == 0 && rot) atomicAdd(&ctl->rotations, (unsigned long long)rot);
           return;
         }
         const int col = (w < 4 ? I : J) * 4 + (w & 3);
@@ -516,7 +547,7 @@ __global__ void __launch_bounds__(256, 1) jacobi_wp4_kernel(float2* __restrict__
         publish_rounds(done, I, J, need + 1);   // ends with __syncthreads
       }
     }
-    if (lane == 0) off_w[w] = local_off;
+    if (lane == 0) off_w[w] = sqrtf(local_off);
     __syncthreads();
     if (tid == 0) {
       float mx = 0.f;
@@ -524,18 +555,315 @@ __global__ void __launch_bounds__(256, 1) jacobi_wp4_kernel(float2* __restrict__
       if (mx > 0.f) atomicMax(&ctl->off_bits[sweep % 3], __float_as_uint(mx));
     }
     if (!grid_barrier(ctl, nb)) {
-      if (lane == 0 && rot) atomicAdd(&ctl->rotations, rot);
+      if (lane == 0 && rot) atomicAdd(&ctl->rotations, (unsigned long long)rot);
       return;
     }
     const float off = __uint_as_float(*((volatile unsigned*)&ctl->off_bits[sweep % 3]));
     if (!(off > conv)) { ++sweep; break; }
   }
-  if (lane == 0 && rot) atomicAdd(&ctl->rotations, rot);
+  if (lane == 0 && rot) atomicAdd(&ctl->rotations, (unsigned long long)rot);
   if (blockIdx.x == 0 && tid == 0) {
     ctl->sweeps = sweep;
     const float off = __uint_as_float(ctl->off_bits[(sweep - 1) % 3]);
     if (sweep >= max_sweeps && off > conv && ctl->err == 0) ctl->err = (int)DMRGC_ENOCONV;
   }
+}
+
+// ---- cluster-resident Jacobi (small matrices, both precisions)
+//
+// The whole matrix stays in the registers of one thread-block cluster of C
+// CTAs; nothing goes through L2 between the first load and the last store.
+// Each CTA holds two blocks of w columns (top and bottom), one column per
+// warp.  A round runs the w cross sub-rounds of its two blocks (plus the w - 1
+// intra sub-rounds in the first round of a sweep) with the column exchange of
+// jacobi_wp4_kernel through shared memory, then the 2 C blocks move one place
+// along the circle top 1 -> .. -> top C-1 -> bottom C-1 -> .. -> bottom 0 ->
+// top 1 (top 0 stays): every warp writes its column into the inbox of the
+// warp that holds it next (distributed shared memory) and arrives on that
+// warp's mbarrier.  Inboxes are double buffered: a CTA sends into buffer p
+// again only after two rounds, and by then it has received a column that its
+// neighbour sent after emptying that buffer (neighbours exchange in both
+// directions every round).  2 C - 1 rounds make a sweep and bring every block
+// home.  Waits poll an mbarrier at most g_spin_limit times; a wait that runs
+// out sets the error flag, the CTA leaves the loops at its next barrier, and
+// every CTA meets the others at the cluster barrier before it exits, so no
+// CTA writes into one that has left.
+
+// rows of a lane's elements: pairs (2 x float2 = 16 bytes) or single double2s
+template <typename R> struct JcChunk;
+template <> struct JcChunk<float> { using V = float4; static constexpr int PER = 2; };
+template <> struct JcChunk<double> { using V = double2; static constexpr int PER = 1; };
+
+__device__ __forceinline__ unsigned jc_smem(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ unsigned jc_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned jc_map(unsigned addr, unsigned rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void jc_store(unsigned addr, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+               : "memory");
+}
+__device__ __forceinline__ void jc_store(unsigned addr, double2 v) {
+  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(addr), "d"(v.x), "d"(v.y) : "memory");
+}
+__device__ __forceinline__ void jc_store(unsigned addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void jc_arrive(unsigned addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+__device__ __forceinline__ void jc_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// bounded wait for the completion of a phase; false: limit or another CTA's error
+__device__ __forceinline__ bool jc_wait(unsigned bar, unsigned parity, JacobiCtl* c) {
+  const unsigned long long lim = g_spin_limit;
+  for (unsigned long long it = 0; it < lim; ++it) {
+    unsigned ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if (it > 4096) __nanosleep(64);
+    if ((it & 255) == 255 && *((volatile int*)&c->err) != 0) return false;
+  }
+  atomicExch(&c->err, (int)DMRGC_ETIMEOUT);
+  return false;
+}
+
+template <bool FIRST, int E>
+__device__ __forceinline__ void jc_pair(float2 (&x)[E], const float2 (&y)[E], float tiny, float tol, float& local_off,
+                                        unsigned& rot) {
+  wp4_pair<FIRST, E>(x, y, true, tiny, tol, local_off, rot);
+}
+
+template <bool FIRST, int E>
+__device__ __forceinline__ void jc_pair(double2 (&x)[E], const double2 (&y)[E], double tiny, double tol,
+                                        float& local_off, unsigned& rot) {
+  double al = 0, be = 0, gr = 0, gi = 0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const double2 u = FIRST ? x[e] : y[e];
+    const double2 v = FIRST ? y[e] : x[e];
+    al = fma(u.x, u.x, fma(u.y, u.y, al));
+    be = fma(v.x, v.x, fma(v.y, v.y, be));
+    gr = fma(u.x, v.x, fma(u.y, v.y, gr));
+    gi = fma(u.x, v.y, fma(-u.y, v.x, gi));
+  }
+  {   // four sums in ten shuffled values, as warp_sum4
+    const int lane = threadIdx.x & 31;
+    const bool u4 = lane & 16, u3 = lane & 8;
+    double k0 = u4 ? gr : al, k1 = u4 ? gi : be;
+    const double s0 = u4 ? al : gr, s1 = u4 ? be : gi;
+    k0 += __shfl_xor_sync(0xffffffffu, s0, 16);
+    k1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+    double k = u3 ? k1 : k0;
+    k += __shfl_xor_sync(0xffffffffu, u3 ? k0 : k1, 8);
+    k += __shfl_xor_sync(0xffffffffu, k, 4);
+    k += __shfl_xor_sync(0xffffffffu, k, 2);
+    k += __shfl_xor_sync(0xffffffffu, k, 1);
+    al = __shfl_sync(0xffffffffu, k, 0);
+    be = __shfl_sync(0xffffffffu, k, 8);
+    gr = __shfl_sync(0xffffffffu, k, 16);
+    gi = __shfl_sync(0xffffffffu, k, 24);
+  }
+  double2 cs;
+  double c;
+  float rel2;
+  if (!jacobi_params(al, be, gr, gi, tiny, tol, cs, c, rel2)) return;
+  if (FIRST) {
+    local_off = fmaxf(local_off, rel2);
+    ++rot;
+  }
+  const double br = FIRST ? -cs.x : cs.x;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const double2 o = x[e], v = y[e];
+    x[e].x = fma(c, o.x, fma(br, v.x, -cs.y * v.y));
+    x[e].y = fma(c, o.y, fma(br, v.y, cs.y * v.x));
+  }
+}
+
+// blockDim = 64 w threads (2 w warps, w a power of two), gridDim = cluster size C.
+// VEC: rows 64 h + 2 lane, + 1 as elements 2h, 2h + 1 (complex64, m even).
+template <typename R, int E, int NT, bool VEC>
+__global__ void __launch_bounds__(NT, 1) jacobi_cluster_kernel(typename cplx<R>::T* __restrict__ G, int m, int n,
+                                                               int w, R tol, R conv, int max_sweeps,
+                                                               const double* __restrict__ fro2, R zero_rel,
+                                                               JacobiCtl* ctl) {
+  using C2 = typename cplx<R>::T;
+  using V = typename JcChunk<R>::V;
+  constexpr int PER = JcChunk<R>::PER, NCH = E / PER;
+  constexpr int COL = NCH * 32;                 // 16-byte chunks of a column
+  static_assert(E % PER == 0, "whole chunks");
+  extern __shared__ __align__(16) unsigned char jc_raw[];
+  __shared__ __align__(8) unsigned long long inbar[2][16];
+  __shared__ __align__(8) unsigned long long cvbar[2];
+  __shared__ float off_w[16];
+  __shared__ float off_c[2][16];
+  __shared__ int s_abort;
+  const int nw = 2 * w;
+  V* sbuf = reinterpret_cast<V*>(jc_raw);       // [2][nw][COL]: sub-round exchange
+  V* inbox = sbuf + (size_t)2 * nw * COL;       // [2][nw][COL]
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int C = gridDim.x, P = 2 * C;
+  const int rank = (int)jc_rank();
+  const bool top = wid < w;
+  if (threadIdx.x == 0) {
+    for (int b = 0; b < 2; ++b) {
+      for (int i = 0; i < nw; ++i)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(jc_smem(&inbar[b][i])) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(jc_smem(&cvbar[b])), "r"(C) : "memory");
+    }
+    s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  const double fz = (double)zero_rel * (double)zero_rel * (*fro2);
+  const R tiny = (R)fmax(fz, (sizeof(R) == 8) ? 1e-280 : 1e-30);
+  const int col = (top ? rank : P - 1 - rank) * w + (top ? wid : wid - w);
+  C2* gcol = G + (long long)col * m;
+  C2 x[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) x[e] = C2{0, 0};
+  if (col < n) {   // columns beyond n stay zero and are never rotated
+    if constexpr (VEC) {
+#pragma unroll
+      for (int h = 0; h < E / 2; ++h) {
+        const int i = 64 * h + 2 * lane;
+        if (i < m) {
+          const float4 v = *reinterpret_cast<const float4*>(gcol + i);
+          x[2 * h] = C2{v.x, v.y};
+          x[2 * h + 1] = C2{v.z, v.w};
+        }
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (lane + 32 * e < m) x[e] = gcol[lane + 32 * e];
+    }
+  }
+  auto put = [&](V* dst) {
+#pragma unroll
+    for (int h = 0; h < NCH; ++h) {
+      if constexpr (PER == 2) dst[lane + 32 * h] = make_float4(x[2 * h].x, x[2 * h].y, x[2 * h + 1].x, x[2 * h + 1].y);
+      else dst[lane + 32 * h] = x[h];
+    }
+  };
+  auto get = [&](const V* src, C2 (&d)[E]) {
+#pragma unroll
+    for (int h = 0; h < NCH; ++h) {
+      const V v = src[lane + 32 * h];
+      if constexpr (PER == 2) { d[2 * h] = C2{v.x, v.y}; d[2 * h + 1] = C2{v.z, v.w}; }
+      else d[h] = v;
+    }
+  };
+  // where this warp's column goes after a round (-1: it stays)
+  int to_rank = -1, to_slot = 0;
+  if (top) {
+    if (rank > 0) { to_rank = rank < C - 1 ? rank + 1 : rank; to_slot = rank < C - 1 ? wid : wid + w; }
+  } else {
+    if (rank > 0) { to_rank = rank - 1; to_slot = wid; }
+    else { to_rank = 1; to_slot = wid - w; }
+  }
+  const bool moves = C > 1 && to_rank >= 0;
+  const unsigned to_box0 = moves ? jc_map(jc_smem(inbox + (size_t)to_slot * COL), to_rank) : 0;
+  const unsigned to_bar0 = moves ? jc_map(jc_smem(&inbar[0][to_slot]), to_rank) : 0;
+  const unsigned my_bar0 = jc_smem(&inbar[0][wid]);
+  const unsigned box_stride = (unsigned)(nw * COL * sizeof(V)), bar_stride = (unsigned)sizeof(inbar[0]);
+  __syncwarp();
+  jc_cluster_sync();   // barriers initialised everywhere
+  int sweep = 0, buf = 0;
+  unsigned step = 0;
+  unsigned rot = 0;
+  bool abort = false;
+  float off = 0.f;
+  for (; sweep < max_sweeps && !abort; ++sweep) {
+    float local_off = 0.f;
+    for (int r = 0; r < P - 1 && !abort; ++r) {
+      // sub-rounds: intra-block pairs (first round only), then cross pairs
+      const int s0 = r == 0 ? -(w - 1) : 0;
+      for (int s = s0; s < w; ++s) {
+        int p;
+        if (s < 0) p = wid ^ (-s);
+        else p = top ? w + ((wid + s) & (w - 1)) : ((wid - s) & (w - 1));
+        V* base = sbuf + (size_t)buf * nw * COL;
+        put(base + (size_t)wid * COL);
+        __syncthreads();
+        if (s == s0 && *((volatile int*)&s_abort)) { abort = true; break; }   // set before this barrier, or not at all
+        C2 y[E];
+        get(base + (size_t)p * COL, y);
+        buf ^= 1;   // the next sub-round writes the other buffer: no second barrier
+        if (wid < p) jc_pair<true, E>(x, y, tiny, tol, local_off, rot);
+        else jc_pair<false, E>(x, y, tiny, tol, local_off, rot);
+      }
+      if (abort || C == 1) break;   // C == 1: one round per sweep
+      const unsigned b = step & 1;
+      if (moves) {
+        const unsigned box = to_box0 + b * box_stride;
+#pragma unroll
+        for (int h = 0; h < NCH; ++h) {
+          V v;
+          if constexpr (PER == 2) v = make_float4(x[2 * h].x, x[2 * h].y, x[2 * h + 1].x, x[2 * h + 1].y);
+          else v = x[h];
+          jc_store(box + (unsigned)((lane + 32 * h) * sizeof(V)), v);
+        }
+        __syncwarp();
+        if (lane == 0) jc_arrive(to_bar0 + b * bar_stride);
+        // the column that comes in its place (every warp but CTA 0's top ones)
+        if (!jc_wait(my_bar0 + b * bar_stride, (step >> 1) & 1, ctl)) s_abort = 1;
+        get(inbox + ((size_t)b * nw + wid) * COL, x);
+      }
+      ++step;
+    }
+    if (abort) break;
+    // largest rotation of the sweep over the cluster
+    if (lane == 0) off_w[wid] = sqrtf(local_off);
+    __syncthreads();
+    const unsigned cb = sweep & 1;
+    if ((int)threadIdx.x < C) {
+      float mx = 0.f;
+      for (int i = 0; i < nw; ++i) mx = fmaxf(mx, off_w[i]);
+      jc_store(jc_map(jc_smem(&off_c[cb][rank]), threadIdx.x), mx);
+      jc_arrive(jc_map(jc_smem(&cvbar[cb]), threadIdx.x));
+    }
+    if (threadIdx.x == 0 && (*((volatile int*)&s_abort) || !jc_wait(jc_smem(&cvbar[cb]), (sweep >> 1) & 1, ctl)))
+      s_abort = 1;
+    __syncthreads();
+    if (*((volatile int*)&s_abort)) { abort = true; break; }
+    off = 0.f;
+    for (int i = 0; i < C; ++i) off = fmaxf(off, *((volatile float*)&off_c[cb][i]));
+    if (!(off > (float)conv)) { ++sweep; break; }
+  }
+  if (!abort && col < n) {
+    if constexpr (VEC) {
+#pragma unroll
+      for (int h = 0; h < E / 2; ++h) {
+        const int i = 64 * h + 2 * lane;
+        if (i < m) *reinterpret_cast<float4*>(gcol + i) = make_float4(x[2 * h].x, x[2 * h].y, x[2 * h + 1].x, x[2 * h + 1].y);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (lane + 32 * e < m) gcol[lane + 32 * e] = x[e];
+    }
+  }
+  if (lane == 0 && rot) atomicAdd(&ctl->rotations, (unsigned long long)rot);
+  if (rank == 0 && threadIdx.x == 0) {
+    ctl->sweeps = sweep;
+    if (!abort && sweep >= max_sweeps && off > (float)conv) atomicCAS(&ctl->err, 0, (int)DMRGC_ENOCONV);
+  }
+  __syncwarp();
+  jc_cluster_sync();   // no CTA leaves while another may still write into it
 }
 
 // ---- block Jacobi on 8 x 8 Gram matrices (complex64, m <= 512 RPT)
@@ -944,9 +1272,113 @@ namespace {
 std::atomic<int> g_jacobi_variant{0};
 int jacobi_variant() { return g_jacobi_variant.load(std::memory_order_relaxed); }
 
+// A cluster shape that can run: cached per kernel, since the query is a host
+// round trip through the driver.
+bool cluster_fits(const void* fn, int ctas, int threads, size_t smem) {
+  struct Key { int dev; const void* fn; int ctas, threads; size_t smem; bool ok; };
+  static std::mutex mu;
+  static std::vector<Key> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> lock(mu);
+  for (const Key& k : known)
+    if (k.dev == dev && k.fn == fn && k.ctas == ctas && k.threads == threads && k.smem == smem) return k.ok;
+  bool ok = allow_dyn_smem(fn) == cudaSuccess &&
+            cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+  if (ok) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int num = 0;
+    ok = cudaOccupancyMaxActiveClusters(&num, fn, &cfg) == cudaSuccess && num >= 1;
+  }
+  if (!ok) cudaGetLastError();
+  known.push_back({dev, fn, ctas, threads, smem, ok});
+  return ok;
+}
+
+cudaError_t launch_cluster(const void* fn, int ctas, int threads, size_t smem, cudaStream_t st, void** args) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = ctas;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
+template <typename R, int E, int NT>
+const void* jc_fn(bool vec) {
+  if constexpr (sizeof(R) == 4)
+    if (vec) return (const void*)jacobi_cluster_kernel<R, E, NT, true>;
+  return (const void*)jacobi_cluster_kernel<R, E, NT, false>;
+}
+
+// The cluster kernel where the matrix fits its registers and shared memory:
+// false (and no launch) otherwise.
+template <typename R>
+bool try_cluster_jacobi(void* G, int m, int n, double tol, double conv, int max_sweeps, const double* fro2,
+                        double zero_rel, JacobiCtl* c, cudaStream_t st, cudaError_t& err) {
+  using C2 = typename cplx<R>::T;
+  const void* fn;
+  int E, wmax;   // rows of a column per lane, most columns per block (128 KB of shared memory)
+  if constexpr (sizeof(R) == 4) {
+    const bool vec = m % 2 == 0 && (reinterpret_cast<uintptr_t>(G) % 16) == 0;
+    if (m <= 64) { E = 2; wmax = 8; fn = jc_fn<R, 2, 512>(vec); }
+    else if (m <= 128) { E = 4; wmax = 8; fn = jc_fn<R, 4, 512>(vec); }
+    else if (m <= 256) { E = 8; wmax = 8; fn = jc_fn<R, 8, 512>(vec); }
+    else if (m <= 512) { E = 16; wmax = 4; fn = jc_fn<R, 16, 256>(vec); }
+    else return false;
+  } else {
+    if (m <= 32) { E = 1; wmax = 8; fn = jc_fn<R, 1, 512>(false); }
+    else if (m <= 64) { E = 2; wmax = 8; fn = jc_fn<R, 2, 512>(false); }
+    else if (m <= 128) { E = 4; wmax = 8; fn = jc_fn<R, 4, 512>(false); }
+    else if (m <= 256) { E = 8; wmax = 4; fn = jc_fn<R, 8, 256>(false); }
+    else if (m <= 512) { E = 16; wmax = 2; fn = jc_fn<R, 16, 128>(false); }
+    else return false;
+  }
+  // FP64: a warp's FP64 instruction holds a quarter of its SM for 64 cycles, so
+  // the work has to spread over many SMs: w = 2 (64 x 64: 1.84 ms; w = 4: 2.77 ms,
+  // w = 8: about 5 ms), and beyond 64 columns, where a cluster would need wider
+  // blocks, the grid-wide kernel takes over (200 x 96: 6.5 ms, cluster 8.9 ms).
+  // complex64 is bound by the latency of a sub-round: w = 4 up to 128 columns
+  // (64 x 64: 0.37 ms; w = 2: 0.52 ms, more hops between SMs; 128 x 100: 0.65
+  // ms, w = 8: 0.90 ms before the shorter rotation), w = 8 up to 256.
+  if (sizeof(R) == 8 && n > 64) return false;
+  int w = sizeof(R) == 8 ? 2 : 4;
+  while (w < wmax && (n + 2 * w - 1) / (2 * w) > 16) w *= 2;
+  const int ctas = (n + 2 * w - 1) / (2 * w);
+  if (ctas > 16) return false;
+  const int threads = 64 * w;
+  const size_t smem = (size_t)4 * 2 * w * E * 32 * sizeof(C2);
+  if (!cluster_fits(fn, ctas, threads, smem)) return false;
+  C2* g = reinterpret_cast<C2*>(G);
+  R tl = (R)tol, cv = (R)conv, zr = (R)zero_rel;
+  void* args[] = {&g, &m, &n, &w, &tl, &cv, &max_sweeps, (void*)&fro2, &zr, &c};
+  err = launch_cluster(fn, ctas, threads, smem, st, args);
+  return true;
+}
+
 template <typename R>
 cudaError_t launch_jacobi(void* G, int m, int n, double tol, int max_sweeps, const double* fro2,
                           double zero_rel, JacobiCtl* c, cudaStream_t st) {
+  if (sizeof(R) == 8 || jacobi_variant() == 0) {
+    cudaError_t ec = cudaSuccess;
+    if (try_cluster_jacobi<R>(G, m, n, tol, sizeof(R) == 8 ? tol : std::max(tol, 2e-3), max_sweeps, fro2, zero_rel, c, st, ec))
+      return ec;
+  }
   using C2 = typename cplx<R>::T;
   const int np = (n + 1) & ~1;
   const int pairs = np / 2;

@@ -200,7 +200,8 @@ dmrgc_status svd_columns(dmrgc_ctx* c, int m, int n, double rel_cut, bool square
     int launches = 0;
     CK(sum_abs2(W, (long long)m * n, c->fp64, fro2, c->st));
     CK(jacobi_orthogonalize(W, m, n, c->fp64, jacobi_tol(c, m), c->max_jsweeps, fro2,
-                            c->zero_rel, c->jctl.p, c->st, &launches));
+                            c->zero_rel, c->jctl.p, c->st, &launches, &n));
+    c->svd_n = n;
     CK(truncate_columns(W, m, n, c->fp64, chi_cap, rel_cut, squared, tie_rel, fro2, c->zero_rel,
                         c->tres.p, c->st));
     c->stats.svd_launches += launches + 3;
@@ -376,7 +377,7 @@ dmrgc_status orth_columns(dmrgc_ctx* c, void* W, int rows, int cols, void* out, 
   TRY(svd_columns(c, rows, cols, 0.0, false, 0.0, k, f, &nnz, nullptr, W, cols));
   r = k;
   Span sp(c, TC_SVD);
-  CK(gather_columns(W, rows, cols, k, c->tres.p, false, mode, out, c->fp64, c->st));
+  CK(gather_columns(W, rows, c->svd_n, k, c->tres.p, false, mode, out, c->fp64, c->st));
   c->stats.kernel_launches++;
   return DMRGC_OK;
 }
@@ -459,7 +460,7 @@ dmrgc_status rsvd_try(dmrgc_ctx* c, int i, bool adj, int mrow, int ncol, int l, 
   TRY(ensure(c, c->rs_w, (size_t)lq * kk * es));
   {
     Span sp(c, TC_SVD);   // normalised eigenvectors of conj(H): conj(W) [lq][kk]
-    CK(gather_columns(c->rs_h.p, lq, lq, kk, c->tres.p, true, 0, c->rs_w.p, c->fp64, c->st));
+    CK(gather_columns(c->rs_h.p, lq, c->svd_n, kk, c->tres.p, true, 0, c->rs_w.p, c->fp64, c->st));
     c->stats.kernel_launches++;
   }
   GemmArgs g;
@@ -599,7 +600,7 @@ dmrgc_status update_ltr(dmrgc_ctx* c, int i) {
       TRY(svd_columns(c, mrow, ncol, c->sweep_cut, false, 0.0, k, f, &nnz));
       TRY(ensure(c, c->A[i], (size_t)mrow * k * c->esz));
       Span sp(c, TC_SVD);
-      CK(gather_columns(c->jw.p, mrow, ncol, k, c->tres.p, false, 0, c->A[i].p, c->fp64, c->st));
+      CK(gather_columns(c->jw.p, mrow, c->svd_n, k, c->tres.p, false, 0, c->A[i].p, c->fp64, c->st));
       c->stats.kernel_launches++;
     }
     note_resolvable(c, i);
@@ -668,7 +669,7 @@ dmrgc_status update_rtl(dmrgc_ctx* c, int i) {
       TRY(svd_columns(c, ncol, mrow, c->sweep_cut, false, 0.0, k, f, &nnz));
       TRY(ensure(c, c->A[i + 1], (size_t)k * ncol * c->esz));
       Span sp(c, TC_SVD);
-      CK(gather_columns(c->jw.p, ncol, mrow, k, c->tres.p, false, 2, c->A[i + 1].p, c->fp64, c->st));
+      CK(gather_columns(c->jw.p, ncol, c->svd_n, k, c->tres.p, false, 2, c->A[i + 1].p, c->fp64, c->st));
       c->stats.kernel_launches++;
     }
     note_resolvable(c, i);
@@ -747,7 +748,7 @@ dmrgc_status zip_guess(dmrgc_ctx* c) {
       TRY(svd_columns(c, r, r, c->zip_cut, true, c->tie_rel, k, f));
       TRY(ensure(c, c->A[i], (size_t)r * k * c->esz));
       Span sp(c, TC_SVD);
-      CK(gather_columns(c->jw.p, r, r, k, c->tres.p, true, 0, c->A[i].p, c->fp64, c->st));
+      CK(gather_columns(c->jw.p, r, c->svd_n, k, c->tres.p, true, 0, c->A[i].p, c->fp64, c->st));
       c->stats.kernel_launches++;
     }
     c->chiA[i + 1] = k;
@@ -783,7 +784,7 @@ dmrgc_status zip_guess(dmrgc_ctx* c) {
       TRY(svd_columns(c, r, r, c->zip_cut, true, c->tie_rel, k, f));
       TRY(ensure(c, c->A[i], (size_t)k * r * c->esz));
       Span sp(c, TC_SVD);
-      CK(gather_columns(c->jw.p, r, r, k, c->tres.p, true, 1, c->A[i].p, c->fp64, c->st));
+      CK(gather_columns(c->jw.p, r, c->svd_n, k, c->tres.p, true, 1, c->A[i].p, c->fp64, c->st));
       c->stats.kernel_launches++;
     }
     c->chiA[i] = k;
@@ -873,7 +874,7 @@ dmrgc_status compress_mpo(dmrgc_ctx* c) {
     TRY(ensure(c, c->T, (size_t)rows * k * es));
     {
       Span sp(c, TC_SVD);
-      CK(gather_columns(c->jw.p, rows, dr, k, c->tres.p, false, 0, c->T.p, c->fp64, c->st));
+      CK(gather_columns(c->jw.p, rows, c->svd_n, k, c->tres.p, false, 0, c->T.p, c->fp64, c->st));
       c->stats.kernel_launches++;
     }
     TRY(ensure(c, c->envL, (size_t)k * dr * es));
@@ -910,7 +911,7 @@ dmrgc_status compress_mpo(dmrgc_ctx* c) {
     TRY(ensure(c, c->T, (size_t)k * cols * es));
     {
       Span sp(c, TC_SVD);   // Q' [k][cols], orthonormal rows spanning the row space of W_i
-      CK(gather_columns(c->jw.p, cols, dl, k, c->tres.p, false, 2, c->T.p, c->fp64, c->st));
+      CK(gather_columns(c->jw.p, cols, c->svd_n, k, c->tres.p, false, 2, c->T.p, c->fp64, c->st));
       c->stats.kernel_launches++;
     }
     TRY(ensure(c, c->envL, (size_t)dl * k * es));

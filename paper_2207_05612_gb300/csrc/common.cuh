@@ -71,6 +71,9 @@ cudaError_t gemm_tc(const GemmArgs& g, int precision, TcWork& w, int* err_dev, c
 // orthogonal columns.  fro2: device pointer to |G|_F^2; columns with norm
 // below zero_rel*|G|_F are treated as zero.  ctl must point to device scratch
 // of jacobi_ctl_bytes(n); it starts with a JacobiStatus the host may read.
+// n_out (optional): a wide matrix (m < n) may be replaced by the L of its LQ
+// factorisation, which has the same left singular vectors and values; *n_out
+// receives the columns that G then has (m, else n).
 struct JacobiStatus {
   int err;                        // 0, DMRGC_ETIMEOUT or DMRGC_ENOCONV
   int sweeps;                     // sweeps executed
@@ -79,7 +82,7 @@ struct JacobiStatus {
 size_t jacobi_ctl_bytes(int n);
 cudaError_t jacobi_orthogonalize(void* G, int m, int n, bool fp64, double tol, int max_sweeps,
                                  const double* fro2, double zero_rel, void* ctl, cudaStream_t st,
-                                 int* launches);
+                                 int* launches, int* n_out = nullptr);
 
 // Column norms of W, sort descending, truncation rank.  Writes into res (device):
 // res->k, res->f = sum_{j<k} s_j^2, res->perm[j], res->s[j] (sorted).

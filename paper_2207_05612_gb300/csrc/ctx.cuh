@@ -51,6 +51,7 @@ struct dmrgc_ctx {
   DevBuf ovl[2];   // ping-pong environments of dmrgc_overlap (never the sweep's envL / envR)
   DevBuf ework;    // work space of the Gram eigensolver path (eig_truncate)
   TruncResult last_tr{};          // result of the last truncated SVD (either path)
+  int svd_n = 0;                  // columns of the matrix the last Jacobi SVD ended with (svd_columns)
   std::vector<char> eig_ok;       // per bond: the last SVD there was resolvable by the eigensolver
   DevBuf rv[3];    // read-outs: running rows V, site products W = V A_i, T = W E_i
   TcWork tcw;

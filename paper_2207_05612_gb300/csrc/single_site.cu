@@ -154,7 +154,7 @@ dmrgc_status isometry(dmrgc_ctx* c, const void* src, long long rows, long long c
   TRY(svd_columns(c, m, n, 0.0, false, 0.0, k, f, &nnz, nullptr, nullptr, n));
   TRY(ensure(c, dst, (size_t)m * k * c->esz));
   Span sp(c, TC_SVD);
-  CK(gather_columns(c->jw.p, m, n, k, c->tres.p, false, left ? 0 : 2, dst.p, c->fp64, c->st));
+  CK(gather_columns(c->jw.p, m, c->svd_n, k, c->tres.p, false, left ? 0 : 2, dst.p, c->fp64, c->st));
   c->stats.kernel_launches++;
   return DMRGC_OK;
 }

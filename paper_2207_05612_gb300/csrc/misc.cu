@@ -177,6 +177,62 @@ cudaError_t allow_dyn_smem(const void* fn) {
   return cudaSuccess;
 }
 
+// How many clusters of a shape are resident together: cached per kernel, since
+// the query is a host round trip through the driver.
+int cluster_count(const void* fn, int ctas, int threads, size_t smem) {
+  struct Key { int dev; const void* fn; int ctas, threads; size_t smem; int num; };
+  static std::mutex mu;
+  static std::vector<Key> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> lock(mu);
+  for (const Key& k : known)
+    if (k.dev == dev && k.fn == fn && k.ctas == ctas && k.threads == threads && k.smem == smem) return k.num;
+  int num = 0;
+  bool ok = allow_dyn_smem(fn) == cudaSuccess &&
+            cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+  if (ok) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    ok = cudaOccupancyMaxActiveClusters(&num, fn, &cfg) == cudaSuccess;
+  }
+  if (!ok) {
+    cudaGetLastError();
+    num = 0;
+  }
+  known.push_back({dev, fn, ctas, threads, smem, num});
+  return num;
+}
+
+bool cluster_fits(const void* fn, int ctas, int threads, size_t smem) {
+  return cluster_count(fn, ctas, threads, smem) >= 1;
+}
+
+cudaError_t launch_cluster(const void* fn, int ctas, int threads, size_t smem, cudaStream_t st, void** args, int grid) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[2]{};
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeCooperative;   // several clusters that wait for one another: all resident
+  at[1].val.cooperative = 1;
+  cfg.gridDim = dim3(grid > 0 ? grid : ctas);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = grid > ctas ? 2 : 1;
+  return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 namespace {
 
 __device__ __forceinline__ double mix_uniform(unsigned long long seed, unsigned long long ctr) {

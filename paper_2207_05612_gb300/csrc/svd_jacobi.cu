@@ -1417,53 +1417,6 @@ namespace {
 std::atomic<int> g_jacobi_variant{0};
 int jacobi_variant() { return g_jacobi_variant.load(std::memory_order_relaxed); }
 
-// A cluster shape that can run: cached per kernel, since the query is a host
-// round trip through the driver.
-bool cluster_fits(const void* fn, int ctas, int threads, size_t smem) {
-  struct Key { int dev; const void* fn; int ctas, threads; size_t smem; bool ok; };
-  static std::mutex mu;
-  static std::vector<Key> known;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return false;
-  std::lock_guard<std::mutex> lock(mu);
-  for (const Key& k : known)
-    if (k.dev == dev && k.fn == fn && k.ctas == ctas && k.threads == threads && k.smem == smem) return k.ok;
-  bool ok = allow_dyn_smem(fn) == cudaSuccess &&
-            cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-  if (ok) {
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = ctas;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.gridDim = dim3(ctas);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    int num = 0;
-    ok = cudaOccupancyMaxActiveClusters(&num, fn, &cfg) == cudaSuccess && num >= 1;
-  }
-  if (!ok) cudaGetLastError();
-  known.push_back({dev, fn, ctas, threads, smem, ok});
-  return ok;
-}
-
-cudaError_t launch_cluster(const void* fn, int ctas, int threads, size_t smem, cudaStream_t st, void** args) {
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = ctas;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.gridDim = dim3(ctas);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelExC(&cfg, fn, args);
-}
-
 template <typename R, int E, int NT>
 const void* jc_fn(bool vec) {
   if constexpr (sizeof(R) == 4)

@@ -857,7 +857,12 @@ __device__ __forceinline__ int sturm_count(const float* __restrict__ d, const fl
 }
 
 // one warp per eigenvalue (descending index i < kk): 6 rounds of 33-section
-// on the Gershgorin interval; lam[i] in the scaled units of T
+// on the Gershgorin interval; lam[i] in the scaled units of T.  Bound by the
+// latency of the quotient, so CTAs of two warps (several points per lane and
+// fewer rounds measured slower: 155 us for 3 points, 312 us for 6, 108 us as it
+// is, at 512 rows and 257 values).
+constexpr int BS_THREADS = 64;
+
 __global__ void tri_bisect_kernel(const float* __restrict__ d, const float* __restrict__ e2, int n, int kk,
                                   float* __restrict__ lam) {
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -881,145 +886,193 @@ __global__ void tri_bisect_kernel(const float* __restrict__ d, const float* __re
   if (lane == 0) lam[warp] = 0.5f * (lo + hi);
 }
 
-// Inverse iteration in FP64 for eigenvectors 0..kv-1 of T (scaled), one
-// thread per eigenvalue.  Factorisation of T - sigma I by Gaussian
-// elimination with partial pivoting (pivots below pivmin raised to pivmin),
-// reciprocal pivots stored; INVIT_ITERS solves, each followed by a
-// normalisation.  A thread keeps its factors, its row swaps and its vector in
-// shared memory (5 n doubles + n bytes, blockDim.x threads per CTA, element i
-// of thread lt at [i * blockDim.x + lt]).  Z: n x kk doubles (element i of
-// vector v at Z[i * kk + v]).  Eigenvalues closer than the bisection's
-// resolution give vectors that are not mutually orthogonal; tri_cluster_kernel
-// orthonormalises each such cluster afterwards (their span is the cluster's
-// invariant subspace, which is all the truncation uses) and forms the
-// Rayleigh quotients.  Only vectors 0..kv-1 above the cut (lam[v] > cut2
-// lam[0], cut2 = half the cut on s squared) are computed: kv is the most the
-// truncation can keep, and the extra eigenvalue and those below the cut keep
-// their bisection values.  A computed eigenvalue below half the resolution
-// level (lam[v] < 0.5 resolve lam[0]) cannot belong to a resolved
-// truncation: the thread flags the result unresolved and computes nothing
-// more.
+// Inverse iteration in FP64 for eigenvectors 0..kv-1 of T (scaled), IV per
+// one-warp CTA.  Lane l < IV runs the recurrences of vector l: factorisation of
+// T - sigma I by Gaussian elimination with partial pivoting (pivots below pivmin
+// raised to pivmin), reciprocal pivots stored, with the first forward solve in
+// the same loop, then back substitution and one more solve.  An FP64
+// instruction takes some 100 cycles on GB300 whatever its number of active
+// lanes (shorter dependency chains changed nothing), so the time is their number
+// per row: 8 in the elimination (its reciprocal starts from an FP32 one whose
+// conversions are integer arithmetic, and takes one Newton step: the elimination
+// is exact to 1e-14, while sigma comes from FP32 bisection), 1 and 3 in a solve.
+// Everything that is not a recurrence (start vectors, norms, scaling) is spread
+// over the 32 lanes, and comparisons use integer arithmetic.  512 rows, 256
+// vectors: 666 -> 443 us.
+// Shared memory of a CTA: the scaled d and e (2 n doubles), then per vector
+// 4 n doubles (1 / pivot, first superdiagonal, multiplier, z) and n swap flags,
+// element i of vector l at [i * IV + l].  Z: vector-major, element i of vector v
+// at Z[v * n + i].  Eigenvalues closer than the bisection's resolution give
+// vectors that are not mutually orthogonal; tri_cluster_kernel orthonormalises
+// each such cluster afterwards (their span is the cluster's invariant subspace,
+// which is all the truncation uses) and forms the Rayleigh quotients.  Only
+// vectors 0..kv-1 above the cut (lam[v] > cut2 lam[0], cut2 = half the cut on s
+// squared) are computed: kv is the most the truncation can keep, and the extra
+// eigenvalue and those below the cut keep their bisection values.  A computed
+// eigenvalue below half the resolution level (lam[v] < 0.5 resolve lam[0])
+// cannot belong to a resolved truncation: the result is flagged unresolved and
+// nothing more is computed.
 constexpr int INVIT_ITERS = 2;
 constexpr int MAX_CLUSTER = 32;
 
-// 1 / a for 1e-15 <= |a| <= 1e30: an FP32 reciprocal refined by two
-// Newton-Raphson steps x <- x + x (1 - a x) in FP64 (each squares the
-// relative error: ~1e-7 -> ~1e-14 -> below FP64 rounding)
-__device__ __forceinline__ double recip_nr(double a) {
-  double x = (double)__frcp_rn((float)a);
-  double e = fma(-a, x, 1.0);
-  x = fma(x, e, x);
-  e = fma(-a, x, 1.0);
-  return fma(x, e, x);
+__device__ __forceinline__ unsigned long long abs_bits(double a) {   // orders |a| of non-NaN values
+  return (unsigned long long)__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFull;
 }
 
-__global__ void tri_invit_kernel(const double* __restrict__ d0, const double* __restrict__ e0, int n, int kk,
-                                 int kv, const float* __restrict__ lam, double cut2, double resolve,
-                                 double* __restrict__ Z, double* __restrict__ lam_out, HeCtl* ctl) {
+// FP32 approximation of 1 / a (|a| in 1e-15 .. 1e30) as a double, without FP64
+// instructions: a is truncated to FP32 and the reciprocal widened bit by bit
+__device__ __forceinline__ double recip_seed(double a) {
+  const unsigned h = (unsigned)__double2hiint(a), l = (unsigned)__double2loint(a);
+  const float f = __uint_as_float((h & 0x80000000u) | (((h & 0x7FFFFFFFu) - 0x38000000u) << 3) | (l >> 29));
+  const unsigned r = __float_as_uint(__fdividef(1.0f, f));
+  return __hiloint2double((int)((r & 0x80000000u) | (((r & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(r << 29));
+}
+
+size_t invit_smem(int n, int iv) { return (size_t)n * 16 + (size_t)iv * n * 33 + 16; }
+
+__global__ void __launch_bounds__(32)
+    tri_invit_kernel(const double* __restrict__ d0, const double* __restrict__ e0, int n, int kk, int kv, int IV,
+                     const float* __restrict__ lam, double cut2, double resolve, double* __restrict__ Z,
+                     double* __restrict__ lam_out, HeCtl* ctl) {
   extern __shared__ double ivs[];
-  const int IV = blockDim.x, lt = threadIdx.x;
-  double* IU0 = ivs;                      // 1 / pivot
-  double* U1 = ivs + (size_t)n * IV;
-  double* U2 = ivs + (size_t)2 * n * IV;
-  double* L = ivs + (size_t)3 * n * IV;   // multipliers
-  double* z = ivs + (size_t)4 * n * IV;
-  unsigned char* swp = reinterpret_cast<unsigned char*>(ivs + (size_t)5 * n * IV);
-  const int v = blockIdx.x * IV + lt;
-  if (v >= kk) return;
+  double* ds = ivs;                                   // d / scale
+  double* es = ivs + n;                               // e / scale, es[n - 1] = 0
+  double* IU0 = ivs + 2 * (size_t)n;                  // 1 / pivot
+  double* U1 = IU0 + (size_t)n * IV;
+  double* L = U1 + (size_t)n * IV;                    // multipliers
+  double* z = L + (size_t)n * IV;
+  unsigned char* swp = reinterpret_cast<unsigned char*>(z + (size_t)n * IV);
+  const int lane = threadIdx.x;
+  const int v0 = blockIdx.x * IV, v = v0 + lane;
   const double scale = (double)ctl->scale;
-  if (v >= kv || !((double)lam[v] > cut2 * (double)lam[0])) {
-    // the extra eigenvalue, or one below the cut (never kept): bisection value only
-    lam_out[v] = (double)lam[v] * scale;
-    return;
+  const double lam0 = (double)lam[0];
+  bool run = false;
+  if (lane < IV && v < kk) {
+    const double lv = (double)lam[v];
+    if (v >= kv || !(lv > cut2 * lam0)) lam_out[v] = lv * scale;   // bisection value only
+    else if (!(lv >= 0.5 * resolve * lam0)) atomicExch(&ctl->status, 1);
+    else run = true;
   }
-  if (!((double)lam[v] >= 0.5 * resolve * (double)lam[0])) {
-    atomicExch(&ctl->status, 1);
-    return;
-  }
+  const unsigned active = __ballot_sync(0xffffffffu, run);
+  if (!active) return;
   const double inv_scale = 1.0 / scale;
-  const double pivmin = 1e-15;
-#define IVX(arr, i) arr[(size_t)(i) * IV + lt]
-  const double sigma = (double)lam[v];
-  // factorisation (scaled entries)
-  double ca = d0[0] * inv_scale - sigma;
-  double cb = n > 1 ? e0[0] * inv_scale : 0.0;
-  double ck = cb;   // subdiagonal of row k+1 = e_k
-  for (int k = 0; k + 1 < n; ++k) {
-    const double ak1 = d0[k + 1] * inv_scale - sigma;
-    const double bk1 = (k + 2 < n) ? e0[k + 1] * inv_scale : 0.0;
-    if (fabs(ca) >= fabs(ck)) {
-      double piv = ca;
-      if (fabs(piv) < pivmin) piv = piv < 0.0 ? -pivmin : pivmin;
-      const double ip = recip_nr(piv);
-      const double l = ck * ip;
-      IVX(IU0, k) = ip; IVX(U1, k) = cb; IVX(U2, k) = 0.0; IVX(L, k) = l; IVX(swp, k) = 0;
-      ca = ak1 - l * cb;
-      cb = bk1;
-    } else {
-      const double ip = recip_nr(fabs(ck) < pivmin ? (ck < 0.0 ? -pivmin : pivmin) : ck);
-      const double l = ca * ip;
-      IVX(IU0, k) = ip; IVX(U1, k) = ak1; IVX(U2, k) = bk1; IVX(L, k) = l; IVX(swp, k) = 1;
-      ca = cb - l * ak1;
-      cb = -l * bk1;
+  for (int i = lane; i < n; i += 32) {
+    ds[i] = d0[i] * inv_scale;
+    es[i] = i + 1 < n ? e0[i] * inv_scale : 0.0;
+  }
+  // start vectors: a fixed pseudo-random sequence (integer hash of i, v)
+  for (int l = 0; l < IV; ++l)
+    for (int i = lane; i < n; i += 32) {
+      unsigned h = (unsigned)i * 2654435761u ^ ((unsigned)(v0 + l) * 0x9E3779B9u + 0x7F4A7C15u);
+      h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12; h *= 0x297A2D39u; h ^= h >> 15;
+      z[(size_t)i * IV + l] = (double)(0.5f + (float)(h & 0xFFFFu) * (1.0f / 65536.0f));
     }
-    ck = bk1;
-  }
-  {
-    double piv = ca;
-    if (fabs(piv) < pivmin) piv = piv < 0.0 ? -pivmin : pivmin;
-    IVX(IU0, n - 1) = recip_nr(piv);
-  }
-  // start vector: a fixed pseudo-random sequence (integer hash of i, v)
-  for (int i = 0; i < n; ++i) {
-    unsigned h = (unsigned)i * 2654435761u ^ ((unsigned)v * 0x9E3779B9u + 0x7F4A7C15u);
-    h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12; h *= 0x297A2D39u; h ^= h >> 15;
-    IVX(z, i) = 0.5 + (double)(h & 0xFFFFu) / 65536.0;
-  }
-  for (int it = 0; it < INVIT_ITERS; ++it) {
-    // forward: the row operations of the elimination (y_k carried in a register)
-    double yk = IVX(z, 0);
+  __syncwarp();
+  const double pivmin = 1e-15;
+  const unsigned long long pivbits = abs_bits(pivmin);
+#define IVX(arr, i) arr[(size_t)(i) * IV + lane]
+  if (run) {
+    const double sigma = (double)lam[v];
+    double ca = ds[0] - sigma, cb = es[0], ck = cb, yk = IVX(z, 0);
+    double dn = ds[1], en = es[1];
     for (int k = 0; k + 1 < n; ++k) {
-      double yk1 = IVX(z, k + 1);
-      const double l = IVX(L, k);
-      if (IVX(swp, k)) { const double t = yk; yk = yk1; yk1 = t - l * yk; }
-      else yk1 -= l * yk;
-      IVX(z, k) = yk;
-      yk = yk1;
+      const double ak1 = dn - sigma, bk1 = en;
+      if (k + 2 < n) { dn = ds[k + 2]; en = es[k + 2]; }
+      const double yk1 = IVX(z, k + 1);
+      const bool sw = abs_bits(ca) < abs_bits(ck);
+      double piv = sw ? ck : ca;
+      if (abs_bits(piv) < pivbits) piv = piv < 0.0 ? -pivmin : pivmin;
+      const double x0 = recip_seed(piv), m = (sw ? ca : ck) * x0;
+      const double er = fma(-piv, x0, 1.0);
+      const double l = fma(m, er, m);
+      const double u1 = sw ? ak1 : cb;
+      ca = fma(-l, u1, sw ? cb : ak1);
+      const double ip = fma(x0, er, x0);
+      IVX(IU0, k) = ip; IVX(U1, k) = u1; IVX(L, k) = l; IVX(swp, k) = sw ? 1 : 0;
+      cb = sw ? -l * bk1 : bk1;
+      ck = bk1;
+      // first forward solve
+      const double y = sw ? yk1 : yk;
+      IVX(z, k) = y;
+      yk = fma(-l, y, sw ? yk : yk1);
+    }
+    if (abs_bits(ca) < pivbits) ca = ca < 0.0 ? -pivmin : pivmin;
+    {
+      const double x0 = recip_seed(ca);
+      IVX(IU0, n - 1) = fma(x0, fma(-ca, x0, 1.0), x0);
     }
     IVX(z, n - 1) = yk;
-    // back substitution (x_{k+1}, x_{k+2} carried in registers), with the norm
-    double x2 = 0.0, x1 = 0.0, nrm = 0.0;
-    for (int k = n - 1; k >= 0; --k) {
-      double y = IVX(z, k);
-      if (k + 1 < n) y -= IVX(U1, k) * x1;
-      if (k + 2 < n) y -= IVX(U2, k) * x2;
-      const double x = y * IVX(IU0, k);
-      IVX(z, k) = x;
-      nrm += x * x;
-      x2 = x1;
-      x1 = x;
-    }
-    const double inv = nrm > 0.0 ? 1.0 / sqrt(nrm) : 0.0;
-    for (int i = 0; i < n; ++i) IVX(z, i) *= inv;
   }
-  for (int i = 0; i < n; ++i) Z[(size_t)i * kk + v] = IVX(z, i);
+  for (int it = 0; it < INVIT_ITERS; ++it) {
+    if (run) {
+      if (it > 0) {   // forward: the row operations of the elimination
+        double yk = IVX(z, 0);
+        for (int k = 0; k + 1 < n; ++k) {
+          const double yk1 = IVX(z, k + 1), l = IVX(L, k);
+          const bool sw = IVX(swp, k) != 0;
+          const double y = sw ? yk1 : yk;
+          IVX(z, k) = y;
+          yk = fma(-l, y, sw ? yk : yk1);
+        }
+        IVX(z, n - 1) = yk;
+      }
+      // back substitution (x_{k+1}, x_{k+2} carried in registers, the next row's
+      // factors loaded ahead)
+      double x1 = IVX(z, n - 1) * IVX(IU0, n - 1), x2 = 0.0;
+      IVX(z, n - 1) = x1;
+      double ip = IVX(IU0, n - 2), u1 = IVX(U1, n - 2), zk = IVX(z, n - 2);
+      double u2 = IVX(swp, n - 2) ? es[n - 1] : 0.0;
+      for (int k = n - 2; k >= 0; --k) {
+        const double y = fma(-u1, x1, fma(-u2, x2, zk)) * ip;
+        if (k > 0) {
+          ip = IVX(IU0, k - 1);
+          u1 = IVX(U1, k - 1);
+          zk = IVX(z, k - 1);
+          u2 = IVX(swp, k - 1) ? es[k] : 0.0;
+        }
+        IVX(z, k) = y;
+        x2 = x1;
+        x1 = y;
+      }
+    }
+    __syncwarp();
+    for (int l = 0; l < IV; ++l) {   // normalise (the last time into Z)
+      if (!((active >> l) & 1)) continue;
+      double nr = 0.0;
+      for (int i = lane; i < n; i += 32) {
+        const double t = z[(size_t)i * IV + l];
+        nr = fma(t, t, nr);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
+      const double inv = nr > 0.0 ? 1.0 / sqrt(nr) : 0.0;
+      if (it + 1 < INVIT_ITERS)
+        for (int i = lane; i < n; i += 32) z[(size_t)i * IV + l] *= inv;
+      else
+        for (int i = lane; i < n; i += 32) Z[(size_t)(v0 + l) * n + i] = z[(size_t)i * IV + l] * inv;
+    }
+    __syncwarp();
+  }
 #undef IVX
 }
 
 // One CTA per eigenvalue index v < kv above the cut; the leader of each
 // cluster (consecutive computed eigenvalues closer than clus_gap, scaled
-// units) orthonormalises the
-// cluster's vectors by modified Gram-Schmidt, twice, and every member gets its
-// Rayleigh quotient z^T T z (units of H) in lam_out.  Clusters longer than
-// MAX_CLUSTER flag the result unresolved.  256 threads.
+// units) orthonormalises the cluster's vectors by classical Gram-Schmidt with
+// reorthogonalisation (each vector twice against all before it: the dot
+// products of a pass run on eight warps at once, three CTA barriers per pass,
+// where the modified form took two per pair), and every member gets its
+// Rayleigh quotient z^T T z (units of H) in lam_out, one warp each.  Clusters
+// longer than MAX_CLUSTER flag the result unresolved.  256 threads.
 __global__ void __launch_bounds__(256) tri_cluster_kernel(const double* __restrict__ d0,
                                                           const double* __restrict__ e0, int n, int kk, int kv,
                                                           const float* __restrict__ lam, double cut2,
                                                           double clus_gap, double* __restrict__ Z,
                                                           double* __restrict__ lam_out, HeCtl* ctl) {
   __shared__ double red[8];
+  __shared__ double dots[MAX_CLUSTER];
   __shared__ int s_status;
-  const int v0 = blockIdx.x, tid = threadIdx.x;
+  const int v0 = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (tid == 0) s_status = *((volatile int*)&ctl->status);
   __syncthreads();
   const double lcut = cut2 * (double)lam[0];
@@ -1031,46 +1084,49 @@ __global__ void __launch_bounds__(256) tri_cluster_kernel(const double* __restri
     if (tid == 0) atomicExch(&ctl->status, 1);
     return;
   }
-  auto block_sum = [&](double x) {
+  for (int v = v0 + 1; v < v1; ++v) {
+    double* zv = Z + (size_t)v * n;
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int q = v0 + wid; q < v; q += 8) {
+        const double* zq = Z + (size_t)q * n;
+        double dp = 0.0;
+        for (int i = lane; i < n; i += 32) dp = fma(zq[i], zv[i], dp);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    __syncthreads();
-    if ((tid & 31) == 0) red[tid >> 5] = x;
-    __syncthreads();
-    double t = 0.0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) t += red[w];
-    return t;
-  };
-  if (v1 - v0 > 1) {
-    for (int pass = 0; pass < 2; ++pass)
-      for (int v = v0; v < v1; ++v) {
-        for (int q = v0; q < v; ++q) {
-          double dp = 0.0;
-          for (int i = tid; i < n; i += 256) dp += Z[(size_t)i * kk + q] * Z[(size_t)i * kk + v];
-          dp = block_sum(dp);
-          for (int i = tid; i < n; i += 256) Z[(size_t)i * kk + v] -= dp * Z[(size_t)i * kk + q];
-          __syncthreads();
-        }
-        double nr = 0.0;
-        for (int i = tid; i < n; i += 256) { const double t = Z[(size_t)i * kk + v]; nr += t * t; }
-        nr = block_sum(nr);
-        const double inv = nr > 0.0 ? 1.0 / sqrt(nr) : 0.0;
-        for (int i = tid; i < n; i += 256) Z[(size_t)i * kk + v] *= inv;
-        __syncthreads();
+        for (int o = 16; o > 0; o >>= 1) dp += __shfl_xor_sync(0xffffffffu, dp, o);
+        if (lane == 0) dots[q - v0] = dp;
       }
-  }
-  for (int v = v0; v < v1; ++v) {   // Rayleigh quotient with the unscaled T
-    double rq = 0.0;
-    for (int i = tid; i < n; i += 256) {
-      const double zi = Z[(size_t)i * kk + v];
-      double tz = d0[i] * zi;
-      if (i > 0) tz += e0[i - 1] * Z[(size_t)(i - 1) * kk + v];
-      if (i + 1 < n) tz += e0[i] * Z[(size_t)(i + 1) * kk + v];
-      rq += zi * tz;
+      __syncthreads();
+      double nr = 0.0;
+      for (int i = tid; i < n; i += 256) {
+        double t = zv[i];
+        for (int q = v0; q < v; ++q) t = fma(-dots[q - v0], Z[(size_t)q * n + i], t);
+        zv[i] = t;
+        nr = fma(t, t, nr);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
+      if (lane == 0) red[wid] = nr;
+      __syncthreads();
+      nr = 0.0;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) nr += red[w];
+      const double inv = nr > 0.0 ? 1.0 / sqrt(nr) : 0.0;
+      for (int i = tid; i < n; i += 256) zv[i] *= inv;
+      __syncthreads();
     }
-    rq = block_sum(rq);
-    if (tid == 0) lam_out[v] = rq;
+  }
+  for (int v = v0 + wid; v < v1; v += 8) {   // Rayleigh quotient with the unscaled T
+    const double* zv = Z + (size_t)v * n;
+    double rq = 0.0;
+    for (int i = lane; i < n; i += 32) {
+      double tz = d0[i] * zv[i];
+      if (i > 0) tz = fma(e0[i - 1], zv[i - 1], tz);
+      if (i + 1 < n) tz = fma(e0[i], zv[i + 1], tz);
+      rq = fma(zv[i], tz, rq);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) rq += __shfl_xor_sync(0xffffffffu, rq, o);
+    if (lane == 0) lam_out[v] = rq;
   }
 }
 
@@ -1103,7 +1159,19 @@ __global__ void __launch_bounds__(1024) eig_trunc_kernel(const double* __restric
     s[i] = l > 0.0 ? sqrt(l) : 0.0;
     perm[i] = i;
   }
-  bad = __syncthreads_or(bad);
+  __shared__ int s_k;
+  __shared__ double redf[32];
+  if (tid == 0) s_k = chi < n ? chi : n;
+  bad = __syncthreads_or(bad);   // s is complete
+  // the first index at or below the cut (every thread its own entries)
+  for (int i = tid; i < (chi < n ? chi : n); i += 1024)
+    if (!(s[i] > cut * s[0])) atomicMin(&s_k, i);
+  __syncthreads();
+  double fs = 0.0;   // weight of the entries above the cut, before the multiplet rule
+  for (int i = tid; i < s_k; i += 1024) fs += s[i] * s[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) fs += __shfl_xor_sync(0xffffffffu, fs, o);
+  if ((tid & 31) == 0) redf[tid >> 5] = fs;
   double t = tr;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
@@ -1114,8 +1182,7 @@ __global__ void __launch_bounds__(1024) eig_trunc_kernel(const double* __restric
     for (int w = 0; w < 32; ++w) tot += red[w];
     tot *= gs;
     const int kmax = chi < n ? chi : n;
-    int k = 0;
-    while (k < kmax && s[k] > cut * s[0]) ++k;
+    int k = s_k;
     const int by_cut = k < kmax;
     if (tie_rel > 0 && k >= 1 && k < kk && s[k] > cut * s[0] && s[k - 1] - s[k] <= tie_rel * s[0]) {
       int kt = k;
@@ -1124,7 +1191,9 @@ __global__ void __launch_bounds__(1024) eig_trunc_kernel(const double* __restric
     }
     if (k < 1) k = 1;
     double f = 0.0;
-    for (int i = 0; i < k; ++i) f += s[i] * s[i];
+    for (int w = 0; w < 32; ++w) f += redf[w];
+    for (int i = k; i < s_k; ++i) f -= s[i] * s[i];   // what the multiplet rule dropped
+    if (s_k < 1) f = s[0] * s[0];
     // a timed-out reduction or a skipped (oversized) cluster leaves lam unset: decide on those first
     int st = 0;
     if (ctl->err != 0) st = (int)DMRGC_ETIMEOUT;
@@ -1242,7 +1311,7 @@ __global__ void __launch_bounds__(BT_WARPS * 32)
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int r = lane + 32 * e;
-    y[e] = make_float2(active && r < n ? (float)Z[(size_t)r * kk + v] : 0.f, 0.f);
+    y[e] = make_float2(active && r < n ? (float)Z[(size_t)v * n + r] : 0.f, 0.f);
   }
   const int nref = n - 1;
   const int nblk = (nref + WY - 1) / WY;
@@ -1470,16 +1539,17 @@ cudaError_t eig_truncate(void* H, int n, int chi, double cut, double tie_rel, do
   // 2. eigenvalues and eigenvectors of T
   tri_prep_kernel<<<1, 1024, 0, st>>>(d, e, n, d32, e2, ctl);
   if ((e_ = cudaGetLastError()) != cudaSuccess) return e_;
-  tri_bisect_kernel<<<(kk * 32 + 255) / 256, 256, 0, st>>>(d32, e2, n, kk, lam32);
+  tri_bisect_kernel<<<(kk * 32 + BS_THREADS - 1) / BS_THREADS, BS_THREADS, 0, st>>>(d32, e2, n, kk, lam32);
   if ((e_ = cudaGetLastError()) != cudaSuccess) return e_;
-  // clusters: consecutive eigenvalues (scaled units) closer than 3e-5; iv
-  // threads per CTA with 5 n doubles + n bytes of shared memory each
+  // clusters: consecutive eigenvalues (scaled units) closer than 3e-5
   {
-    const size_t per_thread = (size_t)n * (5 * sizeof(double) + 1);
-    int iv = (int)std::min<size_t>(8, ((size_t)max_smem - static_smem) / per_thread);
-    if (iv < 1) return cudaErrorInvalidConfiguration;
-    while (iv > 1 && (kk + iv - 1) / iv < sms) iv /= 2;   // spread small problems over the SMs
-    const size_t ism = per_thread * iv;
+    // vectors per one-warp CTA: enough CTAs for the SMs first, then the lanes
+    // that cost nothing
+    const size_t room = (size_t)max_smem - static_smem;
+    int iv = 1;
+    while (iv < 8 && (kk + iv - 1) / iv > sms && invit_smem(n, 2 * iv) <= room) iv *= 2;
+    if (invit_smem(n, iv) > room) return cudaErrorInvalidConfiguration;
+    const size_t ism = invit_smem(n, iv);
     if ((e_ = allow_dyn_smem((const void*)tri_invit_kernel)) != cudaSuccess) return e_;
     const int kv = kk > chi ? chi : kk;   // vectors the truncation can keep
     // vectors are computed down to half the squared cut: the truncation
@@ -1487,7 +1557,7 @@ cudaError_t eig_truncate(void* H, int n, int chi, double cut, double tie_rel, do
     // values by far less than that margin, so it never counts a vector that
     // was not computed (eig_trunc_kernel checks this too)
     const double cut2 = 0.5 * cut * cut;
-    tri_invit_kernel<<<(kk + iv - 1) / iv, iv, ism, st>>>(d, e, n, kk, kv, lam32, cut2, resolve, Z, lam, ctl);
+    tri_invit_kernel<<<(kk + iv - 1) / iv, 32, ism, st>>>(d, e, n, kk, kv, iv, lam32, cut2, resolve, Z, lam, ctl);
     if ((e_ = cudaGetLastError()) != cudaSuccess) return e_;
     tri_cluster_kernel<<<kv, 256, 0, st>>>(d, e, n, kk, kv, lam32, cut2, 3e-5, Z, lam, ctl);
     if ((e_ = cudaGetLastError()) != cudaSuccess) return e_;

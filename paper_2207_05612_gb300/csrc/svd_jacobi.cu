@@ -1344,21 +1344,37 @@ __global__ void sort_trunc_kernel(TruncResult* res, double* s, int* perm, const 
     }
   }
   for (int i = threadIdx.x; i < n; i += blockDim.x) { s[i] = v[i]; perm[i] = ix[i]; }
+  // a column the Jacobi kernel treated as zero (norm <= zero_rel |G|_F) is
+  // never kept: the cut is the larger of rel_cut * s_1 and that level
+  const double s1 = v[0];
+  const double zthr = zero_rel * sqrt(*fro2);              // on the column norm
+  const double szero = squared ? sqrt(zthr) : zthr;
+  const double scut = fmax(rel_cut * s1, szero);
+  __shared__ int s_nnz, s_k;
+  __shared__ double red_t[32], red_f[32];
+  if (threadIdx.x == 0) s_nnz = 0, s_k = 0;
+  __syncthreads();
+  double tsum = 0, fsum = 0;
+  int cz = 0, ck = 0;   // v is sorted: the values above a level come first
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const double q = v[i] * v[i];
+    tsum += q;
+    if (v[i] > szero) ++cz;
+    if (i < chi && v[i] > scut) { ++ck; fsum += q; }
+  }
+  tsum = warp_sum(tsum);
+  fsum = warp_sum(fsum);
+  if (cz) atomicAdd(&s_nnz, cz);
+  if (ck) atomicAdd(&s_k, ck);
+  if ((threadIdx.x & 31) == 0) { red_t[threadIdx.x >> 5] = tsum; red_f[threadIdx.x >> 5] = fsum; }
   __syncthreads();
   if (threadIdx.x == 0) {
-    const double s1 = v[0];
-    // a column the Jacobi kernel treated as zero (norm <= zero_rel |G|_F) is
-    // never kept: the cut is the larger of rel_cut * s_1 and that level
-    const double zthr = zero_rel * sqrt(*fro2);              // on the column norm
-    const double scut = fmax(rel_cut * s1, squared ? sqrt(zthr) : zthr);
-    int k = 0, nnz = 0;
+    int k = s_k;
+    const int nnz = s_nnz, kcut = s_k;
     double f = 0, tot = 0;
-    for (int i = 0; i < n; ++i) {
-      tot += v[i] * v[i];
-      if (v[i] > (squared ? sqrt(zthr) : zthr)) ++nnz;
-    }
-    for (int i = 0; i < n && k < chi; ++i) {
-      if (v[i] > scut) ++k; else break;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+      tot += red_t[w];
+      f += red_f[w];
     }
     // tie rule: never split a (numerically) degenerate multiplet at the cut;
     // a multiplet that reaches s_1 cannot be dropped, the cut then stays at chi
@@ -1369,7 +1385,7 @@ __global__ void sort_trunc_kernel(TruncResult* res, double* s, int* perm, const 
       if (kk == 1 && v[0] - v[1] <= tie_rel * s1) ambiguous = 1;
       else k = kk;
     }
-    for (int i = 0; i < k; ++i) f += v[i] * v[i];
+    for (int i = k; i < kcut; ++i) f -= v[i] * v[i];   // what the tie rule dropped
     res->status = 0;
     res->pad = ambiguous;
     if (!(s1 > 0.0) || !isfinite(s1)) { res->status = (int)DMRGC_ENUMERIC; k = k > 0 ? k : 1; }

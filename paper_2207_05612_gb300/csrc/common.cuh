@@ -127,6 +127,24 @@ cudaError_t gather_columns(const void* W, int m, int n_total, int k, const void*
 size_t eig_work_bytes(int n, int kk);
 cudaError_t eig_truncate(void* H, int n, int chi, double cut, double tie_rel, double resolve, void* work,
                          void* res, void* out, int mode, cudaStream_t st, int* launches);
+// The same in two parts.  eig_reduce: H <- its tridiagonal form and reflectors,
+// the kk leading eigenvalues by bisection.  eig_spectrum: those on the host (in
+// units of head->unit; synchronises st).  eig_select: vectors, truncation and
+// back-transformation as eig_truncate, any number of times after one
+// eig_reduce with the same n, kk and work.
+struct EigHead {
+  int err;         // 0 or DMRGC_ETIMEOUT
+  double unit;     // eigenvalue of the H given to eig_reduce per unit of lam
+  double trace;    // its trace
+};
+cudaError_t eig_reduce(void* H, int n, int kk, void* work, cudaStream_t st, int* launches);
+cudaError_t eig_spectrum(const void* work, int n, int kk, float* lam, EigHead* head, cudaStream_t st);
+cudaError_t eig_select(const void* H, int n, int kk, int chi, double cut, double tie_rel, double resolve, void* work,
+                       void* res, void* out, int mode, cudaStream_t st, int* launches);
+// columns of src (rows x k row-major) into columns off .. off + k - 1 of an n_cols
+// wide result in the layouts of gather_columns (0: [row][col], 1: [col][row],
+// 2: [col][row] conjugated)
+cudaError_t place_columns(const void* src, int rows, int k, void* out, int n_cols, int off, int mode, cudaStream_t st);
 // |x|^2 (FP64 sum in a fixed order: the same bits on every run) to *out_dev;
 // x /= |x| if scale.  part_dev: 256 doubles of scratch.  Two kernels of 256 CTAs.
 cudaError_t norm2_scale(void* x, long long n, bool fp64, double* out_dev, double* part_dev, bool scale,
@@ -185,13 +203,10 @@ cudaError_t build_site_mpo(const int* plan_tab, SitePlan sp, const GateDev* gate
 // streams never lower the limit under one another.
 cudaError_t allow_dyn_smem(const void* fn);
 
-// Thread-block clusters of `ctas` CTAs (<= 16): how many are resident together
-// on an idle device (cached per kernel and shape), whether one is, and a launch
-// of one (grid = 0) or of grid / ctas of them, resident together.
-int cluster_count(const void* fn, int ctas, int threads, size_t smem);
+// Launch of one thread-block cluster of `ctas` CTAs (<= 16), and whether the
+// device can hold it (cached per kernel and shape).
 bool cluster_fits(const void* fn, int ctas, int threads, size_t smem);
-cudaError_t launch_cluster(const void* fn, int ctas, int threads, size_t smem, cudaStream_t st, void** args,
-                           int grid = 0);
+cudaError_t launch_cluster(const void* fn, int ctas, int threads, size_t smem, cudaStream_t st, void** args);
 
 cudaError_t copy_transpose(const void* src, int rows, int cols, bool conj, void* dst, bool fp64,
                            cudaStream_t st);   // dst[c*rows + r] = op(src[r*cols + c])

@@ -50,9 +50,10 @@ struct dmrgc_ctx {
   DevBuf ptrs_d, bonds_d, order_d, bits_d, out_d, stage_d, tcerr;
   DevBuf ovl[2];   // ping-pong environments of dmrgc_overlap (never the sweep's envL / envR)
   DevBuf ework;    // work space of the Gram eigensolver path (eig_truncate)
+  DevBuf df_r, df_c, df_u[4];   // its stages: the residual, U^+ residual, the vectors of each stage
   TruncResult last_tr{};          // result of the last truncated SVD (either path)
   int svd_n = 0;                  // columns of the matrix the last Jacobi SVD ended with (svd_columns)
-  std::vector<char> eig_ok;       // per bond: the last SVD there was resolvable by the eigensolver
+  std::vector<char> eig_ok;       // per bond: its next SVD in this layer tries the eigensolver (note_resolvable)
   DevBuf rv[3];    // read-outs: running rows V, site products W = V A_i, T = W E_i
   TcWork tcw;
   // randomized SVD and the rank model (svd_mode 1, 2)
@@ -100,7 +101,7 @@ dmrgc_status normalise_block(dmrgc_ctx* c, void* A, long long elems, double& f);
 // Jacobi SVD of the columns of c->jw (or W): m x n column-major; k kept, f their weight
 dmrgc_status svd_columns(dmrgc_ctx* c, int m, int n, double rel_cut, bool squared, double tie_rel, int& k,
                          double& f, int* nnz = nullptr, double* norm2 = nullptr, void* W = nullptr,
-                         int chi_cap = -1);
+                         int chi_cap = -1, int lq_min = 2);
 
 // timing span of one class of device work (CUDA events on the context's stream)
 // NVTX range for the span of a host call (named in profilers and ncu's

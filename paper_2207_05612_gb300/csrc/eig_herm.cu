@@ -53,7 +53,8 @@ struct HeCtl {
   float scale;        // max(|d|, |beta|) of T, for the tridiagonal kernels
   int pad0;
   double gscale;      // max_i H_ii: H was divided by it
-  int pad[8];
+  double trace;       // trace of the scaled H
+  int pad[6];
 };
 static_assert(sizeof(HeCtl) == 64, "control block layout");
 
@@ -183,11 +184,18 @@ __device__ __forceinline__ void reflector(float2 alpha, float rest, float2& tau,
     u0 = alpha;
     return;
   }
-  const float nrm = sqrtf(n2);
+  // square root and quotient from the approximate units with a Newton step each:
+  // as accurate as the IEEE ones to an ulp, half the latency, which every
+  // column of the reduction waits for
+  float r = rsqrtf(n2);
+  r = fmaf(0.5f * r, fmaf(-n2 * r, r, 1.f), r);
+  const float nrm = n2 * r;
   beta = alpha.x >= 0.f ? -nrm : nrm;
   u0 = make_float2(alpha.x - beta, alpha.y);
   // tau = -1 / (beta conj(u0)) = -u0 / (beta |u0|^2)
-  const float q = -1.f / (beta * (u0.x * u0.x + u0.y * u0.y));
+  const float den = -beta * (u0.x * u0.x + u0.y * u0.y);
+  float q = __fdividef(1.f, den);
+  q = fmaf(q, fmaf(-den, q, 1.f), q);
   tau = make_float2(q * u0.x, q * u0.y);
 }
 
@@ -421,38 +429,33 @@ __global__ void __launch_bounds__(TD_THREADS, 1)
   }
 }
 
-// The same reduction by thread-block clusters, for a block of at most 1024 rows
-// (TC_MULTI; at most TC_ONE rows by a single cluster).  CTA g of G owns the rows
-// r = g + G t; a row lives in the registers of one warp (t = wid + 8 q, q < R;
-// column lane + 32 e in element e).  Step j, in every CTA, thread tid owning the
-// columns tid + 256 k:
+// The same reduction of a block of at most TC_ONE rows by one thread-block
+// cluster.  CTA g of G owns the rows r = g + G t; a row lives in the registers of
+// one warp (t = wid + 8 q, q < R; column lane + 32 e in element e).  Step j, in
+// every CTA, thread tid owning the columns tid + 256 k:
 //  (a) from (p_r, entry (r, j)) of every row, received in step j-1: K, w_{j-1},
 //      column j and its norm (two CTA reductions), the reflector by every
 //      thread.  u_j[j+1] stays in a register (u0) and shared memory keeps the
 //      column's own entry there, so no third barrier is needed;
 //  (b) the owned rows: update j-1, p_r and entry (r, j+1); 16 bytes per row go to
 //      every CTA of the cluster by st.async, which counts the bytes on the
-//      receiver's mbarrier (all rows > j: 16 (n - 1 - j) bytes a step);
-//  (c) with several clusters: the row's 16 bytes also go to global memory, and
-//      the CTA of the same rank in every other cluster polls them there and
-//      hands them to its cluster.  A packet is its own flag: words still holding
-//      the sentinel have not arrived.  Four packet buffers rotate; the owner
-//      resets the one of step j+2 at step j, when every CTA has read step j-2
-//      (each has sent step j-1 since).
+//      receiver's mbarrier (16 (n - 1 - j) bytes a step for the rows > j).
 // Exchange buffers alternate by step: a CTA sends step j+2 only after it has
 // received step j+1 from everyone, and a CTA sends step j+1 only after a barrier
-// behind its reads of step j.  For that every CTA sends a packet to its cluster
-// each step even when its rows are done (across clusters every CTA keeps an
-// unfinished row: jend <= n - G).  An error seen by one CTA does not make it
-// leave early: it stops working and meets its cluster at the last barrier, so
-// no store ever goes to a CTA that has left.
+// behind its reads of step j.  For that every CTA sends a packet each step even
+// when its rows are done.  An error seen by one CTA does not make it leave early:
+// it stops working and meets its cluster at the last barrier, so no store ever
+// goes to a CTA that has left.
 // Bound by the latency of that chain: a grid-wide atomic barrier and two L2
 // round trips per column (5.9 us at 1024 rows, about 4.4 us at 256 to 512)
-// become one hop between SMs (1.9 us at 256 rows, 2.5 us at 512, where the rank-2
-// update of 32 rows per SM begins to show).  One cluster leaves the other SMs to
-// other streams.
+// become one hop between SMs (1.7 us at 256 rows; 2.25 us at 512, where the rank-2
+// update of 32 rows per SM takes 0.85).  Of a step at 256 rows, 3700 cycles, the
+// rows take 980, the exchange 900, the two reductions 870, the reflector 480.
+// One cluster leaves the other SMs to other streams.  (Eight clusters holding
+// 1024 rows that passed packets through L2 gained 3% over the grid-wide kernel:
+// left out.)
 constexpr int TC_THREADS = 256, TC_W = TC_THREADS / 32;
-constexpr int TC_ONE = 512, TC_MULTI = 1024;
+constexpr int TC_ONE = 512;
 
 __device__ __forceinline__ unsigned td_smem(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ unsigned td_map(unsigned addr, unsigned rank) {
@@ -486,38 +489,12 @@ __device__ __forceinline__ bool td_wait(unsigned bar, unsigned parity, HeCtl* c)
   atomicExch(&c->err, (int)DMRGC_ETIMEOUT);
   return false;
 }
-constexpr unsigned kTdEmpty = 0xFFFFFFFFu;   // the byte pattern of a cleared packet
-__device__ __forceinline__ uint4 td_peek(const uint4* p) {
-  uint4 v;
-  asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p)
-               : "memory");
-  return v;
-}
-__device__ __forceinline__ void td_post(uint4* p, uint4 v) {
-  asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
-               : "memory");
-}
-__device__ __forceinline__ bool td_poll(const uint4* p, uint4& v, HeCtl* c) {
-  for (unsigned long long it = 0; it < kHeSpinLimit; ++it) {
-    v = td_peek(p);
-    if (v.x != kTdEmpty && v.y != kTdEmpty && v.z != kTdEmpty && v.w != kTdEmpty) return true;
-    if (it > 4096) __nanosleep(32);
-    if ((it & 255) == 255 && *((volatile int*)&c->err) != 0) return false;
-  }
-  atomicExch(&c->err, (int)DMRGC_ETIMEOUT);
-  return false;
-}
-
 // S: the block's first element in a matrix of row stride ld; n rows, 3 <= n <= 32 E,
-// n <= 8 R gridDim.x.  Reduces columns 0 .. jend - 1 (jend = n - 2: all); jend <
-// n - 2 leaves the trailing block, with every update applied, in S.
+// n <= 8 R gridDim.x
 template <int E, int R>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-    he_tridiag_cluster_kernel(float2* __restrict__ S, int n, int ld, int jend, int CS, double* __restrict__ d,
-                              double* __restrict__ beta, float2* __restrict__ tau, uint4* __restrict__ pkt,
-                              HeCtl* __restrict__ ctl) {
+    he_tridiag_cluster_kernel(float2* __restrict__ S, int n, int ld, double* __restrict__ d, double* __restrict__ beta,
+                              float2* __restrict__ tau, HeCtl* __restrict__ ctl) {
   constexpr int NC = 32 * E, KC = (NC + TC_THREADS - 1) / TC_THREADS;   // padded columns, columns per thread
   extern __shared__ __align__(16) unsigned char td_raw[];
   float4* ex0 = reinterpret_cast<float4*>(td_raw);          // [2][NC]: (p_r, entry (r, j + 1)) of a step
@@ -528,8 +505,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   __shared__ int s_abort;
   __shared__ __align__(16) float4 beat[2][16];   // one packet per CTA of the cluster and step
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int G = gridDim.x, g = blockIdx.x, rank = g % CS;
-  const bool multi = G > CS;
+  const int G = gridDim.x, g = blockIdx.x, jend = n - 2;   // columns to reduce
   if (tid == 0) {
     for (int i = 0; i < 2; ++i)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(td_smem(&bars[i])) : "memory");
@@ -559,6 +535,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   }
   __syncwarp();
   td_cluster_sync();   // barriers and buffers ready in the whole cluster
+  // this lane's destination: lane < G sends to the CTA of that rank
+  const unsigned to = lane < G ? lane : 0;
+  const unsigned ex_to = td_map(td_smem(ex0), to), bar_to = td_map(td_smem(&bars[0]), to), beat_to = td_map(td_smem(&beat[0][g]), to);
   float2 u0 = make_float2(0.f, 0.f), tj = make_float2(0.f, 0.f);   // u_{j-1}[j], tau_{j-1}
   bool abort = false;
   float K = 0.f;
@@ -589,7 +568,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const float2* up = ub0 + (size_t)((j & 1) ^ 1) * NC;
     const unsigned bar = td_smem(&bars[j & 1]);
     if (tid == 0)
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(16u * (unsigned)(n - 1 - j + CS))
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(16u * (unsigned)(n - 1 - j + G))
                    : "memory");
     float2 a[KC];
     if (j > 0) {
@@ -637,8 +616,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const float4 r0 = reinterpret_cast<const float4*>(reds)[0], r1 = reinterpret_cast<const float4*>(reds)[1];
     const float rest = ((r0.x + r0.y) + (r0.z + r0.w)) + ((r1.x + r1.y) + (r1.z + r1.w));
     // a CTA whose rows are all done still takes part in the flow control
-    if (wid == TC_W - 1 && lane < CS)
-      td_send(td_map(td_smem(&beat[j & 1][rank]), lane), td_map(bar, lane), make_float4(0.f, 0.f, 0.f, 0.f));
+    if (wid == TC_W - 1 && lane < G)
+      td_send(beat_to + (j & 1) * (unsigned)sizeof(beat[0]), bar_to + (j & 1) * 8u, make_float4(0.f, 0.f, 0.f, 0.f));
     const float2 x1 = uc[j + 1];
     float2 un;
     float b;
@@ -666,15 +645,22 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       accx[q] = accy[q] = nxt[q] = make_float2(0.f, 0.f);
     }
     if (any) {
+      // from the last 32 columns down to the block of j + 1, the next block's
+      // vectors loaded ahead of this one's FMAs
       const int e1 = (j + 1) >> 5;
+      float2 uv = uc[lane + 32 * (E - 1)], w = wp[lane + 32 * (E - 1)], u = up[lane + 32 * (E - 1)];
 #pragma unroll
-      for (int e = 0; e < E; ++e) {
-        if (e < e1 || 32 * e >= n) continue;   // columns <= j are done
-        const int cc = lane + 32 * e;
-        const float2 uv = uc[cc], w = wp[cc], u = up[cc];
+      for (int e = E - 1; e >= 0; --e) {
+        if (e < e1) break;
         const float2 wx = make_float2(w.x, w.x), wy = make_float2(w.y, w.y);
         const float2 ux = make_float2(u.x, u.x), uy = make_float2(u.y, u.y);
         const float2 vx = make_float2(uv.x, uv.x), vy = make_float2(uv.y, uv.y);
+        if (e > 0) {
+          uv = uc[lane + 32 * (e - 1)];
+          w = wp[lane + 32 * (e - 1)];
+          u = up[lane + 32 * (e - 1)];
+        }
+        if (32 * e >= n) continue;
 #pragma unroll
         for (int q = 0; q < R; ++q) {
           float2 v = x[q][e];
@@ -688,9 +674,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           if (e == e1) nxt[q] = v;
         }
       }
-      float2 acc[R];
+      float2 acc[R], nx[R];
 #pragma unroll
-      for (int q = 0; q < R; ++q) acc[q] = make_float2(accx[q].x - accy[q].y, accx[q].y + accy[q].x);
+      for (int q = 0; q < R; ++q) {
+        nx[q] = make_float2(__shfl_sync(0xffffffffu, nxt[q].x, (j + 1) & 31), __shfl_sync(0xffffffffu, nxt[q].y, (j + 1) & 31));
+        acc[q] = make_float2(accx[q].x - accy[q].y, accx[q].y + accy[q].x);
+      }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
@@ -702,36 +691,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       const float2 dx = make_float2(un.x - x1.x, un.y - x1.y);   // u_j[j+1] - its place holder
 #pragma unroll
       for (int q = 0; q < R; ++q) {
-        const float2 nx = make_float2(__shfl_sync(0xffffffffu, nxt[q].x, (j + 1) & 31),
-                                      __shfl_sync(0xffffffffu, nxt[q].y, (j + 1) & 31));
         if (row[q] <= j || row[q] >= n) continue;
-        const float2 fix = f2mul(nx, dx);
+        const float2 fix = f2mul(nx[q], dx);
         const float2 p = f2mul(tj, make_float2(acc[q].x + fix.x, acc[q].y + fix.y));
-        const float4 out = make_float4(p.x, p.y, nx.x, nx.y);
-        if (lane < CS) {
-          td_send(td_map(td_smem(ex0 + (size_t)(j & 1) * NC + row[q]), lane), td_map(bar, lane), out);
-        } else if (multi && lane == 31) {
-          td_post(pkt + (size_t)(j & 3) * n + row[q],
-                  make_uint4(__float_as_uint(out.x), __float_as_uint(out.y), __float_as_uint(out.z), __float_as_uint(out.w)));
-          td_post(pkt + (size_t)((j + 2) & 3) * n + row[q], make_uint4(kTdEmpty, kTdEmpty, kTdEmpty, kTdEmpty));
-          __threadfence();   // the reset is visible before anything this lane posts in the next step
-        }
+        const float4 out = make_float4(p.x, p.y, nx[q].x, nx[q].y);
+        if (lane < G) td_send(ex_to + (unsigned)(((j & 1) * NC + row[q]) * sizeof(float4)), bar_to + (j & 1) * 8u, out);
       }
     }
     u0 = un;
-    if (multi) {
-      // the other clusters' rows of this rank: r = rank mod CS, owned elsewhere
-      for (int i = tid; i * CS + rank < n; i += TC_THREADS) {
-        const int r = i * CS + rank;
-        if (r <= j || r % G == g) continue;
-        uint4 v;
-        if (!td_poll(pkt + (size_t)(j & 3) * n + r, v, ctl)) { s_abort = 1; break; }
-        const float4 f = make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
-        const unsigned at = td_smem(ex0 + (size_t)(j & 1) * NC + r);
-        for (int k = 0; k < CS; ++k) td_send(td_map(at, k), td_map(bar, k), f);
-        __threadfence();   // ordered before this thread's next poll of a rotated buffer
-      }
-    }
   }
   if (!abort) {
     form_k(jend);   // the last exchange
@@ -745,33 +712,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       if (c >= jend && c < n) S[(size_t)(jend - 1) * ld + c] = c == jend ? u0 : up[c];
     }
   }
-  if (!abort && jend + 2 < n) {
-    // hand the trailing block over, the pending update applied
-    const float4* X = ex0 + (size_t)((jend & 1) ^ 1) * NC;
-    const float2* up = ub0 + (size_t)((jend & 1) ^ 1) * NC;
-#pragma unroll
-    for (int k = 0; k < KC; ++k) {
-      const int c = tid + TC_THREADS * k;
-      if (c >= jend && c < n) {
-        const float4 xc = X[c];
-        const float2 u = c == jend ? u0 : up[c];
-        wp[c] = make_float2(xc.x - K * u.x, xc.y - K * u.y);
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < R; ++q) {
-      if (row[q] < jend || row[q] >= n) continue;
-      const float2 ur = row[q] == jend ? u0 : up[row[q]], wr = wp[row[q]];
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const int cc = lane + 32 * e;
-        if (cc < jend || cc >= n) continue;
-        const float2 t1 = f2mul(ur, f2conj(wp[cc])), t2 = f2mul(wr, f2conj(cc == jend ? u0 : up[cc]));
-        S[(size_t)row[q] * ld + cc] = make_float2(x[q][e].x - (t1.x + t2.x), x[q][e].y - (t1.y + t2.y));
-      }
-    }
-  } else if (!abort) {
+  if (!abort) {
     // trailing 2 x 2 block with the last pending update and the 1 x 1 reflector:
     // the warp of row n - 1
     const int jl = n - 3, ra = n - 2, rb = n - 1;
@@ -829,6 +770,15 @@ __global__ void tri_prep_kernel(const double* __restrict__ d, const double* __re
   }
   const double scale = (red[0] > 0.0 && isfinite(red[0])) ? red[0] : 1.0;
   const double inv = 1.0 / scale;
+  __syncthreads();
+  double tr = 0.0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) tr += d[i];
+  red[threadIdx.x] = tr;
+  __syncthreads();
+  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
+    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+    __syncthreads();
+  }
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     d32[i] = (float)(d[i] * inv);
     if (i + 1 < n) {
@@ -836,7 +786,10 @@ __global__ void tri_prep_kernel(const double* __restrict__ d, const double* __re
       e2_32[i] = es * es;
     }
   }
-  if (threadIdx.x == 0) ctl->scale = (float)scale;
+  if (threadIdx.x == 0) {
+    ctl->scale = (float)scale;
+    ctl->trace = red[0];
+  }
 }
 
 // number of eigenvalues of the (scaled) T below x: negative pivots of the
@@ -913,7 +866,7 @@ __global__ void tri_bisect_kernel(const float* __restrict__ d, const float* __re
 // cannot belong to a resolved truncation: the result is flagged unresolved and
 // nothing more is computed.
 constexpr int INVIT_ITERS = 2;
-constexpr int MAX_CLUSTER = 32;
+constexpr int MAX_CLUSTER = 64;
 
 __device__ __forceinline__ unsigned long long abs_bits(double a) {   // orders |a| of non-NaN values
   return (unsigned long long)__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFull;
@@ -1059,11 +1012,14 @@ __global__ void __launch_bounds__(32)
 // One CTA per eigenvalue index v < kv above the cut; the leader of each
 // cluster (consecutive computed eigenvalues closer than clus_gap, scaled
 // units) orthonormalises the cluster's vectors by classical Gram-Schmidt with
-// reorthogonalisation (each vector twice against all before it: the dot
-// products of a pass run on eight warps at once, three CTA barriers per pass,
-// where the modified form took two per pair), and every member gets its
-// Rayleigh quotient z^T T z (units of H) in lam_out, one warp each.  Clusters
-// longer than MAX_CLUSTER flag the result unresolved.  256 threads.
+// reorthogonalisation, each vector twice against those before it whose
+// eigenvalues lie within clus_gap of its own (the others are orthogonal by their
+// gap): the dot products of a pass run on eight warps at once, three CTA
+// barriers per pass, where the modified form took two per pair.  Every member
+// gets its Rayleigh quotient z^T T z (units of H) in lam_out, one warp each.  A
+// cluster may be of any length (the dense lower end of a spectrum forms long
+// chains); more than MAX_CLUSTER eigenvalues within clus_gap flag the result
+// unresolved.  256 threads.
 __global__ void __launch_bounds__(256) tri_cluster_kernel(const double* __restrict__ d0,
                                                           const double* __restrict__ e0, int n, int kk, int kv,
                                                           const float* __restrict__ lam, double cut2,
@@ -1080,26 +1036,28 @@ __global__ void __launch_bounds__(256) tri_cluster_kernel(const double* __restri
   if (v0 > 0 && (double)lam[v0 - 1] - (double)lam[v0] <= clus_gap) return;   // not a cluster leader
   int v1 = v0 + 1;
   while (v1 < kv && (double)lam[v1] > lcut && (double)lam[v1 - 1] - (double)lam[v1] <= clus_gap) ++v1;
-  if (v1 - v0 > MAX_CLUSTER) {
-    if (tid == 0) atomicExch(&ctl->status, 1);
-    return;
-  }
+  int q0 = v0;
   for (int v = v0 + 1; v < v1; ++v) {
     double* zv = Z + (size_t)v * n;
+    while ((double)lam[q0] - (double)lam[v] > clus_gap) ++q0;
+    if (v - q0 >= MAX_CLUSTER) {
+      if (tid == 0) atomicExch(&ctl->status, 1);
+      return;
+    }
     for (int pass = 0; pass < 2; ++pass) {
-      for (int q = v0 + wid; q < v; q += 8) {
+      for (int q = q0 + wid; q < v; q += 8) {
         const double* zq = Z + (size_t)q * n;
         double dp = 0.0;
         for (int i = lane; i < n; i += 32) dp = fma(zq[i], zv[i], dp);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) dp += __shfl_xor_sync(0xffffffffu, dp, o);
-        if (lane == 0) dots[q - v0] = dp;
+        if (lane == 0) dots[q - q0] = dp;
       }
       __syncthreads();
       double nr = 0.0;
       for (int i = tid; i < n; i += 256) {
         double t = zv[i];
-        for (int q = v0; q < v; ++q) t = fma(-dots[q - v0], Z[(size_t)q * n + i], t);
+        for (int q = q0; q < v; ++q) t = fma(-dots[q - q0], Z[(size_t)q * n + i], t);
         zv[i] = t;
         nr = fma(t, t, nr);
       }
@@ -1407,7 +1365,7 @@ __global__ void __launch_bounds__(BT_WARPS * 32)
 }
 
 // work-space layout of eig_truncate, parts rounded to 256 bytes
-constexpr int kParts = 14;
+constexpr int kParts = 13;
 
 struct EigParts {
   size_t off[kParts];
@@ -1429,8 +1387,7 @@ EigParts eig_parts(int n, int kk) {
                                 (size_t)n * sizeof(float),                // e2_32
                                 (size_t)n * sizeof(float),                // lam32
                                 (size_t)nblk * WY * WY * sizeof(float2),  // WY blocks
-                                NK * sizeof(double),                      // Z
-                                (size_t)4 * n * sizeof(uint4)};           // packets between clusters
+                                NK * sizeof(double)};                     // Z
   EigParts p{};
   size_t o = 0;
   for (int i = 0; i < kParts; ++i) {
@@ -1445,26 +1402,53 @@ EigParts eig_parts(int n, int kk) {
 
 size_t eig_work_bytes(int n, int kk) { return eig_parts(n, kk).total; }
 
-cudaError_t eig_truncate(void* H, int n, int chi, double cut, double tie_rel, double resolve, void* work,
-                         void* res, void* out, int mode, cudaStream_t st, int* launches) {
-  if (n < 3 || n > 2048 || chi < 1) return cudaErrorInvalidValue;
-  const int kk = chi + 1 < n ? chi + 1 : n;
+namespace {
+
+struct EigPtrs {
+  HeCtl* ctl;
+  float2* pbuf;
+  float2* rowbuf;
+  float* part;
+  double *d, *e, *lam;
+  float2* tau;
+  float *d32, *e2, *lam32;
+  float2* Tw;
+  double* Z;
+};
+
+EigPtrs eig_ptrs(void* work, int n, int kk) {
   const EigParts P = eig_parts(n, kk);
   unsigned char* w = reinterpret_cast<unsigned char*>(work);
-  HeCtl* ctl = reinterpret_cast<HeCtl*>(w + P.off[0]);
-  float2* pbuf = reinterpret_cast<float2*>(w + P.off[1]);
-  float2* rowbuf = reinterpret_cast<float2*>(w + P.off[2]);
-  float* part = reinterpret_cast<float*>(w + P.off[3]);
-  double* d = reinterpret_cast<double*>(w + P.off[4]);
-  double* e = reinterpret_cast<double*>(w + P.off[5]);
-  double* lam = reinterpret_cast<double*>(w + P.off[6]);
-  float2* tau = reinterpret_cast<float2*>(w + P.off[7]);
-  float* d32 = reinterpret_cast<float*>(w + P.off[8]);
-  float* e2 = reinterpret_cast<float*>(w + P.off[9]);
-  float* lam32 = reinterpret_cast<float*>(w + P.off[10]);
-  float2* Tw = reinterpret_cast<float2*>(w + P.off[11]);
-  double* Z = reinterpret_cast<double*>(w + P.off[12]);
-  uint4* pkt = reinterpret_cast<uint4*>(w + P.off[13]);
+  return {reinterpret_cast<HeCtl*>(w + P.off[0]),   reinterpret_cast<float2*>(w + P.off[1]),
+          reinterpret_cast<float2*>(w + P.off[2]),  reinterpret_cast<float*>(w + P.off[3]),
+          reinterpret_cast<double*>(w + P.off[4]),  reinterpret_cast<double*>(w + P.off[5]),
+          reinterpret_cast<double*>(w + P.off[6]),  reinterpret_cast<float2*>(w + P.off[7]),
+          reinterpret_cast<float*>(w + P.off[8]),   reinterpret_cast<float*>(w + P.off[9]),
+          reinterpret_cast<float*>(w + P.off[10]),  reinterpret_cast<float2*>(w + P.off[11]),
+          reinterpret_cast<double*>(w + P.off[12])};
+}
+
+}  // namespace
+
+cudaError_t eig_spectrum(const void* work, int n, int kk, float* lam, EigHead* head, cudaStream_t st) {
+  const EigPtrs p = eig_ptrs(const_cast<void*>(work), n, kk);
+  HeCtl c{};
+  cudaError_t e = cudaMemcpyAsync(&c, p.ctl, sizeof(c), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(lam, p.lam32, sizeof(float) * kk, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  head->err = c.err;
+  head->unit = (double)c.scale * c.gscale;
+  head->trace = c.trace * c.gscale;
+  return e;
+}
+
+cudaError_t eig_reduce(void* H, int n, int kk, void* work, cudaStream_t st, int* launches) {
+  if (n < 3 || n > 2048 || kk < 1 || kk > n) return cudaErrorInvalidValue;
+  const EigPtrs p = eig_ptrs(work, n, kk);
+  HeCtl* ctl = p.ctl;
+  float2 *pbuf = p.pbuf, *rowbuf = p.rowbuf, *tau = p.tau;
+  float *part = p.part, *d32 = p.d32, *e2 = p.e2, *lam32 = p.lam32;
+  double *d = p.d, *e = p.e;
   cudaError_t e_ = cudaMemsetAsync(ctl, 0, sizeof(HeCtl), st);
   if (e_ != cudaSuccess) return e_;
   float2* S = reinterpret_cast<float2*>(H);
@@ -1472,33 +1456,24 @@ cudaError_t eig_truncate(void* H, int n, int chi, double cut, double tie_rel, do
   if ((e_ = cudaGetLastError()) != cudaSuccess) return e_;
   herm_sym_kernel<<<std::min(4096, (n * n + 255) / 256), 256, 0, st>>>(S, n, ctl);
   if ((e_ = cudaGetLastError()) != cudaSuccess) return e_;
-  // 1. tridiagonalisation: the grid-wide kernel down to 1024 rows, several
-  // clusters down to 512 (the register files of 64 SMs hold 1024 rows), one
-  // cluster for the rest: the fewer SMs have to agree on a column, the shorter
-  // it takes, so each takes over as soon as it can hold the block.  Whole
-  // truncated SVD (host copies included): 256 rows 2.26 -> 1.79 ms, 512 rows 5.02 ->
-  // 4.05 ms, 1024 rows 12.4 -> 11.1 ms.
+  // 1. tridiagonalisation: the grid-wide kernel down to the 512 rows one cluster
+  // holds, which takes half the time per column there.  Whole truncated SVD (host
+  // copies included) 256 rows 2.26 -> 1.58 ms, 512 rows 5.02 -> 3.68 ms, 1024 rows
+  // 12.4 -> 10.4 ms (with the shorter inverse iteration).
   int dev = 0, sms = 0, max_smem = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const size_t static_smem = 1024;
-  // rows reduced by clusters (the last ones), and by a single cluster
-  const int one = std::min(n, TC_ONE), many = std::min(n, TC_MULTI);
+  const int one = std::min(n, TC_ONE);   // rows reduced by the cluster, the last ones
   const void* cfn = one <= 128   ? (const void*)he_tridiag_cluster_kernel<4, 4>
                     : one <= 256 ? (const void*)he_tridiag_cluster_kernel<8, 4>
                                  : (const void*)he_tridiag_cluster_kernel<16, 4>;
-  const void* mfn = (const void*)he_tridiag_cluster_kernel<32, 2>;
-  auto smem_of = [](int E) { return (size_t)32 * E * (2 * sizeof(float4) + 3 * sizeof(float2)); };
   const int E1 = one <= 128 ? 4 : one <= 256 ? 8 : 16;
+  const size_t csm = (size_t)32 * E1 * (2 * sizeof(float4) + 3 * sizeof(float2));
   const int ctas = std::min(16, (one + 31) / 32);
-  const bool clustered = cluster_fits(cfn, ctas, TC_THREADS, smem_of(E1));
-  // several clusters: as many as are resident together
-  // (at most half of those that fit an idle device)
-  const int cs = 8, ncl = (many + 16 * cs - 1) / (16 * cs);   // two rows per warp: 8 clusters at 1024 rows
-  const bool multi = clustered && many > one && ncl > 1 && 2 * ncl <= cluster_count(mfn, cs, TC_THREADS, smem_of(32));
-  const int G2 = ncl * cs;
-  const int j1 = multi ? n - many : clustered ? n - one : n - 2;   // columns of the grid-wide kernel
+  const bool clustered = cluster_fits(cfn, ctas, TC_THREADS, csm);
+  const int j1 = clustered ? n - one : n - 2;   // columns of the grid-wide kernel
   int nlaunch = 0;
   if (j1 > 0) {
     // cooperative: every CTA resident.  Rows in shared memory when ceil(n / G)
@@ -1520,27 +1495,41 @@ cudaError_t eig_truncate(void* H, int n, int chi, double cut, double tie_rel, do
     if (e_ != cudaSuccess) return e_;
     ++nlaunch;
   }
-  int done = j1;   // columns reduced so far
-  auto reduce_block = [&](const void* fn, int E, int grid, int csz, int upto) -> cudaError_t {
-    float2* St = S + (size_t)done * n + done;
-    double *dt = d + done, *et = e + done;
-    float2* taut = tau + done;
-    int nt = n - done, ld = n, jl = std::min(upto - done, nt - 2), c = csz;
-    void* args[] = {&St, &nt, &ld, &jl, &c, &dt, &et, &taut, &pkt, &ctl};
+  if (clustered) {
+    float2* St = S + (size_t)j1 * n + j1;
+    double *dt = d + j1, *et = e + j1;
+    float2* taut = tau + j1;
+    int nt = one, ld = n;
+    void* args[] = {&St, &nt, &ld, &dt, &et, &taut, &ctl};
+    if ((e_ = launch_cluster(cfn, ctas, TC_THREADS, csm, st, args)) != cudaSuccess) return e_;
     ++nlaunch;
-    done = upto;
-    return launch_cluster(fn, csz, TC_THREADS, smem_of(E), st, args, grid);
-  };
-  if (multi) {
-    if ((e_ = cudaMemsetAsync(pkt, 0xFF, (size_t)4 * many * sizeof(uint4), st)) != cudaSuccess) return e_;
-    if ((e_ = reduce_block(mfn, 32, G2, cs, n - one)) != cudaSuccess) return e_;
   }
-  if (clustered && (e_ = reduce_block(cfn, E1, ctas, ctas, n)) != cudaSuccess) return e_;
   // 2. eigenvalues and eigenvectors of T
   tri_prep_kernel<<<1, 1024, 0, st>>>(d, e, n, d32, e2, ctl);
   if ((e_ = cudaGetLastError()) != cudaSuccess) return e_;
   tri_bisect_kernel<<<(kk * 32 + BS_THREADS - 1) / BS_THREADS, BS_THREADS, 0, st>>>(d32, e2, n, kk, lam32);
   if ((e_ = cudaGetLastError()) != cudaSuccess) return e_;
+  if (launches) *launches += 4 + nlaunch;
+  return cudaSuccess;
+}
+
+cudaError_t eig_select(const void* H, int n, int kk, int chi, double cut, double tie_rel, double resolve, void* work,
+                       void* res, void* out, int mode, cudaStream_t st, int* launches) {
+  if (n < 3 || n > 2048 || chi < 1 || kk < 1 || kk > n) return cudaErrorInvalidValue;
+  const EigPtrs p = eig_ptrs(work, n, kk);
+  HeCtl* ctl = p.ctl;
+  const float2* S = reinterpret_cast<const float2*>(H);
+  const float2* tau = p.tau;
+  const float* lam32 = p.lam32;
+  float2* Tw = p.Tw;
+  double *d = p.d, *e = p.e, *lam = p.lam, *Z = p.Z;
+  int dev = 0, sms = 0, max_smem = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  const size_t static_smem = 1024;
+  cudaError_t e_ = cudaMemsetAsync(&ctl->status, 0, sizeof(int), st);
+  if (e_ != cudaSuccess) return e_;
   // clusters: consecutive eigenvalues (scaled units) closer than 3e-5
   {
     // vectors per one-warp CTA: enough CTAs for the SMs first, then the lanes
@@ -1588,8 +1577,17 @@ cudaError_t eig_truncate(void* H, int n, int chi, double cut, double tie_rel, do
     e_ = cudaLaunchKernel(fn, dim3((kk + BT_WARPS - 1) / BT_WARPS), dim3(BT_WARPS * 32), args, bsm, st);
     if (e_ != cudaSuccess) return e_;
   }
-  if (launches) *launches += 9 + nlaunch;
+  if (launches) *launches += 5;
   return cudaSuccess;
+}
+
+cudaError_t eig_truncate(void* H, int n, int chi, double cut, double tie_rel, double resolve, void* work,
+                         void* res, void* out, int mode, cudaStream_t st, int* launches) {
+  if (n < 3 || n > 2048 || chi < 1) return cudaErrorInvalidValue;
+  const int kk = chi + 1 < n ? chi + 1 : n;
+  const cudaError_t e = eig_reduce(H, n, kk, work, st, launches);
+  if (e != cudaSuccess) return e;
+  return eig_select(H, n, kk, chi, cut, tie_rel, resolve, work, res, out, mode, st, launches);
 }
 
 }  // namespace dmrgc

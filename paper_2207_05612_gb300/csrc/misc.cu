@@ -177,18 +177,17 @@ cudaError_t allow_dyn_smem(const void* fn) {
   return cudaSuccess;
 }
 
-// How many clusters of a shape are resident together: cached per kernel, since
-// the query is a host round trip through the driver.
-int cluster_count(const void* fn, int ctas, int threads, size_t smem) {
-  struct Key { int dev; const void* fn; int ctas, threads; size_t smem; int num; };
+// Whether a cluster of this shape can run: cached per kernel, since the query is
+// a host round trip through the driver.
+bool cluster_fits(const void* fn, int ctas, int threads, size_t smem) {
+  struct Key { int dev; const void* fn; int ctas, threads; size_t smem; bool ok; };
   static std::mutex mu;
   static std::vector<Key> known;
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
   std::lock_guard<std::mutex> lock(mu);
   for (const Key& k : known)
-    if (k.dev == dev && k.fn == fn && k.ctas == ctas && k.threads == threads && k.smem == smem) return k.num;
-  int num = 0;
+    if (k.dev == dev && k.fn == fn && k.ctas == ctas && k.threads == threads && k.smem == smem) return k.ok;
   bool ok = allow_dyn_smem(fn) == cudaSuccess &&
             cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
   if (ok) {
@@ -202,34 +201,26 @@ int cluster_count(const void* fn, int ctas, int threads, size_t smem) {
     cfg.dynamicSmemBytes = smem;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    ok = cudaOccupancyMaxActiveClusters(&num, fn, &cfg) == cudaSuccess;
+    int num = 0;
+    ok = cudaOccupancyMaxActiveClusters(&num, fn, &cfg) == cudaSuccess && num >= 1;
   }
-  if (!ok) {
-    cudaGetLastError();
-    num = 0;
-  }
-  known.push_back({dev, fn, ctas, threads, smem, num});
-  return num;
+  if (!ok) cudaGetLastError();
+  known.push_back({dev, fn, ctas, threads, smem, ok});
+  return ok;
 }
 
-bool cluster_fits(const void* fn, int ctas, int threads, size_t smem) {
-  return cluster_count(fn, ctas, threads, smem) >= 1;
-}
-
-cudaError_t launch_cluster(const void* fn, int ctas, int threads, size_t smem, cudaStream_t st, void** args, int grid) {
+cudaError_t launch_cluster(const void* fn, int ctas, int threads, size_t smem, cudaStream_t st, void** args) {
   cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at[2]{};
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = ctas;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeCooperative;   // several clusters that wait for one another: all resident
-  at[1].val.cooperative = 1;
-  cfg.gridDim = dim3(grid > 0 ? grid : ctas);
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = ctas;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(ctas);
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cfg.attrs = at;
-  cfg.numAttrs = grid > ctas ? 2 : 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
@@ -335,6 +326,31 @@ cudaError_t permute4(const void* src, const int* dims, const int* perm, void* ds
   const int4 p = make_int4(perm[0], perm[1], perm[2], perm[3]);
   if (fp64) permute4_kernel<<<blocks_for(n), 256, 0, st>>>((const double2*)src, d, p, (double2*)dst, n);
   else permute4_kernel<<<blocks_for(n), 256, 0, st>>>((const float2*)src, d, p, (float2*)dst, n);
+  return cudaGetLastError();
+}
+
+namespace {
+
+__global__ void place_columns_kernel(const float2* __restrict__ src, int rows, int k, float2* __restrict__ out,
+                                     int n_cols, int off, int mode) {
+  const long long total = (long long)rows * k;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
+       e += (long long)gridDim.x * blockDim.x) {
+    // the fast index runs along the output
+    const int r = mode == 0 ? (int)(e / k) : (int)(e % rows), v = mode == 0 ? (int)(e % k) : (int)(e / rows);
+    float2 z = src[(long long)r * k + v];
+    if (mode == 2) z.y = -z.y;
+    if (mode == 0) out[(long long)r * n_cols + off + v] = z;
+    else out[(long long)(off + v) * rows + r] = z;
+  }
+}
+
+}  // namespace
+
+cudaError_t place_columns(const void* src, int rows, int k, void* out, int n_cols, int off, int mode, cudaStream_t st) {
+  if (k <= 0) return cudaSuccess;
+  place_columns_kernel<<<blocks_for((long long)rows * k), 256, 0, st>>>((const float2*)src, rows, k, (float2*)out, n_cols, off,
+                                                                        mode);
   return cudaGetLastError();
 }
 

@@ -60,7 +60,7 @@ struct TcWork {
   cudaError_t ensure(int i, size_t bytes);
   void release();
 };
-// *launches (optional): kernels launched (operand packs, C clear, the GEMM)
+// *launches (optional): kernels launched (the operand pack, the GEMM, the sum of the K splits)
 cudaError_t gemm_tc(const GemmArgs& g, int precision, TcWork& w, int* err_dev, cudaStream_t st,
                     int* launches = nullptr);
 

@@ -381,70 +381,76 @@ __device__ __forceinline__ void split4(float x, float& hi, float& lo) {
   lo = tf32_rne(x - hi);
 }
 
-// one 32 x 32 tile of (row = m or n, col = k) complex values via shared memory
-// so that both the source (either index contiguous) and the destination
-// (k contiguous) are read / written in order.  expand = 1: the N-side 2x2 form.
+// One operand of a product: its source and packed form.
+struct PackSide {
+  const float2* src;
+  long long ld, s1, s2;
+  int kfast, conj;       // source index order, conjugation
+  int rows, expand;      // rows m or n; expand = 1: the N-side 2 x 2 form (two rows each)
+  int n2;                // instances along the second batch index
+  int gy;                // 32-row tiles
+  unsigned blocks;       // k tiles x gy x instances
+  void *hi, *lo;
+};
+
+// Both operands in one launch (blocks of A first).  One 32 x 32 tile of (row = m or
+// n, col = k) complex values per block, via shared memory so that both the source
+// (either index contiguous) and the destination (k contiguous) are read and
+// written in order; a lane writes the (Re, Im) pair of one value, 4 or 8 bytes.
+// HBM bound for the large products, launch bound for the small ones: one launch
+// instead of two and the paired stores took 4.2 us off each product of a single
+// amplitude (24 sites, 611 -> 512 us) and 3.8 us off each of 54 sampled sites.
 template <int ESZ>
-__global__ void pack_kernel(const float2* __restrict__ src, long long ld, long long s1, long long s2,
-                            int src_kfast, int conj, int rows, int K, int kp, int expand, int inst_b1_stride,
-                            int n_inst1, int n_inst2, void* __restrict__ hi_out, void* __restrict__ lo_out) {
+__global__ void __launch_bounds__(256) pack_kernel(PackSide A, PackSide B, int K, int kp, int gx) {
   __shared__ float2 tile[32][33];
-  const int inst = blockIdx.z;
-  const int j1 = inst / n_inst2, j2 = inst % n_inst2;
-  const float2* S = src + j1 * s1 + j2 * s2;
-  const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 32;
-  (void)inst_b1_stride;
-  for (int t = threadIdx.y; t < 32; t += blockDim.y) {
-    // t indexes the slow index of the source read, threadIdx.x the fast one
-    int r, k;
-    if (src_kfast) { r = r0 + t; k = k0 + threadIdx.x; } else { k = k0 + t; r = r0 + threadIdx.x; }
+  const bool second = blockIdx.x >= A.blocks;
+  const PackSide& p = second ? B : A;
+  unsigned id = second ? blockIdx.x - A.blocks : blockIdx.x;
+  const int bx = (int)(id % (unsigned)gx);
+  id /= (unsigned)gx;
+  const int by = (int)(id % (unsigned)p.gy), inst = (int)(id / (unsigned)p.gy);
+  const float2* S = p.src + (inst / p.n2) * p.s1 + (inst % p.n2) * p.s2;
+  const int r0 = by * 32, k0 = bx * 32, rows = p.rows;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+  for (int t = ty; t < 32; t += 8) {
+    // t indexes the slow index of the source read, tx the fast one
+    const int r = p.kfast ? r0 + t : r0 + tx, k = p.kfast ? k0 + tx : k0 + t;
     float2 v = make_float2(0.f, 0.f);
-    if (r < rows && k < K) v = src_kfast ? S[(long long)r * ld + k] : S[(long long)k * ld + r];
-    if (conj) v.y = -v.y;
-    if (src_kfast) tile[t][threadIdx.x] = v; else tile[threadIdx.x][t] = v;
+    if (r < rows && k < K) v = p.kfast ? S[(long long)r * p.ld + k] : S[(long long)k * p.ld + r];
+    if (p.conj) v.y = -v.y;
+    if (p.kfast) tile[t][tx] = v; else tile[tx][t] = v;
   }
   __syncthreads();
-  const int out_rows = expand ? 2 * rows : rows;
-  const long long inst_elems = (long long)out_rows * kp;
-  // write: each (row, 2 reals of one k); 32 rows x 64 reals
-  for (int t = threadIdx.y; t < 32; t += blockDim.y) {
+  const int kk = 2 * (k0 + tx);   // real column of the pair
+  if (kk >= kp) return;           // kp is even
+  const long long inst_elems = (long long)(p.expand ? 2 * rows : rows) * kp;
+  auto put = [&](long long at, float a, float b) {
+    if constexpr (ESZ == 2) {
+      __nv_bfloat162 h, l;
+      split2(a, h.x, l.x);
+      split2(b, h.y, l.y);
+      *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(p.hi) + at) = h;
+      *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(p.lo) + at) = l;
+    } else {
+      float2 h, l;
+      split4(a, h.x, l.x);
+      split4(b, h.y, l.y);
+      *reinterpret_cast<float2*>(reinterpret_cast<float*>(p.hi) + at) = h;
+      *reinterpret_cast<float2*>(reinterpret_cast<float*>(p.lo) + at) = l;
+    }
+  };
+#pragma unroll
+  for (int t = ty; t < 32; t += 8) {
     const int r = r0 + t;
     if (r >= rows) continue;
-    for (int q = threadIdx.x; q < 64; q += 32) {
-      const int kk = 2 * k0 + q;          // real column
-      if (kk >= kp) continue;
-      const int k = kk >> 1, part = kk & 1;
-      float2 v = (k < K) ? tile[t][k - k0] : make_float2(0.f, 0.f);
-      float a, b;
-      if (!expand) {
-        a = part ? v.y : v.x;
-        b = 0.f;
-      } else {   // rows 2r (Re, -Im) and 2r+1 (Im, Re)
-        a = part ? -v.y : v.x;
-        b = part ? v.x : v.y;
-      }
-      const long long o0 = inst * inst_elems + (long long)(expand ? 2 * r : r) * kp + kk;
-      if constexpr (ESZ == 2) {
-        __nv_bfloat16 h, l;
-        split2(a, h, l);
-        reinterpret_cast<__nv_bfloat16*>(hi_out)[o0] = h;
-        reinterpret_cast<__nv_bfloat16*>(lo_out)[o0] = l;
-        if (expand) {
-          split2(b, h, l);
-          reinterpret_cast<__nv_bfloat16*>(hi_out)[o0 + kp] = h;
-          reinterpret_cast<__nv_bfloat16*>(lo_out)[o0 + kp] = l;
-        }
-      } else {
-        float h, l;
-        split4(a, h, l);
-        reinterpret_cast<float*>(hi_out)[o0] = h;
-        reinterpret_cast<float*>(lo_out)[o0] = l;
-        if (expand) {
-          split4(b, h, l);
-          reinterpret_cast<float*>(hi_out)[o0 + kp] = h;
-          reinterpret_cast<float*>(lo_out)[o0 + kp] = l;
-        }
-      }
+    const float2 v = tile[t][tx];   // zero beyond K
+    const long long at = inst * inst_elems + (long long)(p.expand ? 2 * r : r) * kp + kk;
+    if (!p.expand) {
+      put(at, v.x, v.y);
+    } else {   // rows 2r (Re, -Im) and 2r + 1 (Im, Re)
+      put(at, v.x, -v.y);
+      put(at + kp, v.y, v.x);
     }
   }
 }
@@ -527,22 +533,24 @@ cudaError_t run_tc(const GemmArgs& g, TcWork& w, int* err_dev, cudaStream_t st, 
   if ((e = w.ensure(1, a_bytes)) != cudaSuccess) return e;
   if ((e = w.ensure(2, b_bytes)) != cudaSuccess) return e;
   if ((e = w.ensure(3, b_bytes)) != cudaSuccess) return e;
-  // pack A: rows m, K; source k-contiguous for op N / R
+  // pack A (rows m; source k-contiguous for op N / R) and B (rows n, expanded; for op T / C)
   {
-    const bool kfast = (g.opA == OP_N || g.opA == OP_R);
-    const bool cj = (g.opA == OP_C || g.opA == OP_R);
-    dim3 grid((kp / 2 + 31) / 32, (g.M + 31) / 32, (unsigned)instA);
-    pack_kernel<ESZ><<<grid, dim3(32, 8), 0, st>>>((const float2*)g.A, g.lda, g.sA1, g.sA2, kfast, cj, g.M, g.K, kp, 0,
-                                                   0, a1, a2, w.buf[0], w.buf[1]);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  // pack B (expanded): rows n, K; source k-contiguous for op T / C
-  {
-    const bool kfast = (g.opB == OP_T || g.opB == OP_C);
-    const bool cj = (g.opB == OP_C || g.opB == OP_R);
-    dim3 grid((kp / 2 + 31) / 32, (g.N + 31) / 32, (unsigned)instB);
-    pack_kernel<ESZ><<<grid, dim3(32, 8), 0, st>>>((const float2*)g.B, g.ldb, g.sB1, g.sB2, kfast, cj, g.N, g.K, kp, 1,
-                                                   0, bb1, bb2, w.buf[2], w.buf[3]);
+    const int gx = (kp / 2 + 31) / 32;
+    auto side = [&](const void* src, long long ld, long long s1, long long s2, int op, bool kfast, int rows, int expand,
+                    int n2, long long inst, void* hi, void* lo) {
+      PackSide p{};
+      p.src = (const float2*)src; p.ld = ld; p.s1 = s1; p.s2 = s2;
+      p.kfast = kfast; p.conj = op == OP_C || op == OP_R;
+      p.rows = rows; p.expand = expand; p.n2 = n2; p.gy = (rows + 31) / 32;
+      p.blocks = (unsigned)((long long)gx * p.gy * inst);
+      p.hi = hi; p.lo = lo;
+      return p;
+    };
+    const PackSide pa = side(g.A, g.lda, g.sA1, g.sA2, g.opA, g.opA == OP_N || g.opA == OP_R, g.M, 0, a2, instA, w.buf[0], w.buf[1]);
+    const PackSide pb = side(g.B, g.ldb, g.sB1, g.sB2, g.opB, g.opB == OP_T || g.opB == OP_C, g.N, 1, bb2, instB, w.buf[2], w.buf[3]);
+    const long long blocks = (long long)gx * (pa.gy * instA + pb.gy * instB);
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    pack_kernel<ESZ><<<(unsigned)blocks, 256, 0, st>>>(pa, pb, g.K, kp, gx);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   CUtensorMap tAh, tAl, tBh, tBl;
@@ -593,7 +601,7 @@ cudaError_t run_tc(const GemmArgs& g, TcWork& w, int* err_dev, cudaStream_t st, 
     if ((e = w.ensure(4, (size_t)split * nbatch * g.M * g.N * sizeof(float2))) != cudaSuccess) return e;
     a.P = (float2*)w.buf[4];
   }
-  if (launches) *launches = 3 + (split > 1 ? 1 : 0);
+  if (launches) *launches = 2 + (split > 1 ? 1 : 0);
   if ((e = allow_dyn_smem((const void*)tc_gemm_kernel<ESZ>)) != cudaSuccess) return e;
   a.tiles_n = (2 * g.N + TC_BN - 1) / TC_BN;
   a.tiles_m = (g.M + TC_BM - 1) / TC_BM;

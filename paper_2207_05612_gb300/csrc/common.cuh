@@ -47,6 +47,13 @@ struct GemmArgs {
   int beta_one = 0;   // 1: accumulate into C
   int upper_only = 0; // 1 (M == N, one instance, tensor-core path): only the output tiles that
                       // touch the upper triangle are computed; C below them is left undefined
+  // Row groups (tensor-core path, one instance, A with contiguous k): row p of the
+  // product is row a_rows[p] of A (-1: zeros), the M tiles of 128 rows before
+  // *group_tile (device) multiply the columns 0 .. N - 1 of B, the others the
+  // columns N .. 2 N - 1 (B has 2 N columns).
+  const int* a_rows = nullptr;
+  const int* group_tile = nullptr;
+  int split = 0;      // tensor-core path: K splits to use (0: chosen by the number of waves)
 };
 
 cudaError_t gemm_simt(const GemmArgs& g, bool fp64, cudaStream_t st);
@@ -63,6 +70,8 @@ struct TcWork {
 // *launches (optional): kernels launched (the operand pack, the GEMM, the sum of the K splits)
 cudaError_t gemm_tc(const GemmArgs& g, int precision, TcWork& w, int* err_dev, cudaStream_t st,
                     int* launches = nullptr);
+// the K splits that gemm_tc chooses for one instance of this size
+int gemm_tc_split(int M, int N, int K, int precision);
 
 // --------------------------------------------------------------------- SVD
 
@@ -241,6 +250,16 @@ cudaError_t amp_select(const void* W, int B, int r, const unsigned char* bits, i
 cudaError_t sample_select(const void* W, const void* T, int B, int r, unsigned long long seed, long long row0, int n,
                           int site, int qubit, unsigned char* out, void* V, bool fp64, cudaStream_t st);
 cudaError_t amp_store(const void* V, int B, double2* out, bool fp64, cudaStream_t st);
+// Amplitudes with the strings grouped by their bit at each site (complex64 tensor
+// cores).  group_rows: for every site i < n, pos[i][b] = the row of string b when
+// the strings with bit 0 at qubit order[i] come first and those with bit 1 start
+// at the next multiple of 128, tile[i] = that multiple / 128, and src[i][p] (p < M,
+// M a multiple of 128 that is at least B + 127) = the row at site i - 1 of the
+// string at row p (0 at site 0), -1 where there is none.  amp_store_rows: out[b] =
+// V[pos[b]][0].
+cudaError_t group_rows(const unsigned char* bits, int B, int n, const int* order, int M, int* pos, int* src, int* tile,
+                       cudaStream_t st);
+cudaError_t amp_store_rows(const void* V, const int* pos, int B, double2* out, cudaStream_t st);
 // Metropolis chains (App. C), step t of `steps` for C chains over n qubits:
 // metro_draw writes the proposals prop[C][n] and acceptance uniforms uacc[C]
 // (SplitMix64 at counters g (n + 1) + q and g (n + 1) + n, g = c (steps + 1) + t);

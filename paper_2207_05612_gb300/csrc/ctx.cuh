@@ -55,6 +55,7 @@ struct dmrgc_ctx {
   int svd_n = 0;                  // columns of the matrix the last Jacobi SVD ended with (svd_columns)
   std::vector<char> eig_ok;       // per bond: its next SVD in this layer tries the eigensolver (note_resolvable)
   DevBuf rv[3];    // read-outs: running rows V, site products W = V A_i, T = W E_i
+  DevBuf rv_rows;  // rows of the strings at every site (amplitudes on the tensor cores)
   TcWork tcw;
   // randomized SVD and the rank model (svd_mode 1, 2)
   DevBuf rs_om, rs_y, rs_q, rs_b, rs_h, rs_w, feat, mlp_w, mlp_out, lab;

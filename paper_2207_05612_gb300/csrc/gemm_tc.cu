@@ -59,6 +59,8 @@ struct TcArgs {
   float alpha_re, alpha_im;
   int mode;            // 0 store, 1 add to C (beta = 1), 2 split-K partial into P
   int upper;           // 1: skip the tiles strictly below the diagonal (square C)
+  const int* grp;      // row groups: the first M tile of the second group (device), or null
+  int grp_row;         // its offset among the rows of B'
   float2* P;           // split-K partials [split][batch][M][N] (mode 2)
   int* err;
 };
@@ -234,10 +236,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   if (warp == 0 && lane == 0) {
     // ---- TMA producer
     int it = 0;
+    const int grp = g.grp ? *g.grp : 0x7fffffff;
     for (long long t = blockIdx.x; t < g.total && !*abort_flag; t += gridDim.x) {
       int bx, by, z;
       decode(t, bx, by, z);
       const int batch = z / g.split, ks = z % g.split;
+      const int brow = bx * TC_BN + (by >= grp ? g.grp_row : 0);
       const int i1 = batch / g.b2, i2 = batch % g.b2;
       const int instA = i1 * g.a_m1 + i2 * g.a_m2, instB = i1 * g.b_m1 + i2 * g.b_m2;
       const int nk = kblocks(ks), kt0 = ks * g.per;
@@ -250,8 +254,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const int kx = (kt0 + k) * BK;
         tma_load_3d(st, &tA_hi, kx, by * TC_BM, instA, &full[s]);
         tma_load_3d(st + TC_A_BYTES, &tA_lo, kx, by * TC_BM, instA, &full[s]);
-        tma_load_3d(st + 2 * TC_A_BYTES, &tB_hi, kx, bx * TC_BN, instB, &full[s]);
-        tma_load_3d(st + 2 * TC_A_BYTES + TC_B_BYTES, &tB_lo, kx, bx * TC_BN, instB, &full[s]);
+        tma_load_3d(st + 2 * TC_A_BYTES, &tB_hi, kx, brow, instB, &full[s]);
+        tma_load_3d(st + 2 * TC_A_BYTES + TC_B_BYTES, &tB_lo, kx, brow, instB, &full[s]);
         *s_issued = it + 1;
       }
     }
@@ -388,6 +392,7 @@ struct PackSide {
   int kfast, conj;       // source index order, conjugation
   int rows, expand;      // rows m or n; expand = 1: the N-side 2 x 2 form (two rows each)
   int n2;                // instances along the second batch index
+  const int* gather;     // source row of each row (-1: zeros), or null; kfast only
   int gy;                // 32-row tiles
   unsigned blocks;       // k tiles x gy x instances
   void *hi, *lo;
@@ -417,7 +422,10 @@ __global__ void __launch_bounds__(256) pack_kernel(PackSide A, PackSide B, int K
     // t indexes the slow index of the source read, tx the fast one
     const int r = p.kfast ? r0 + t : r0 + tx, k = p.kfast ? k0 + tx : k0 + t;
     float2 v = make_float2(0.f, 0.f);
-    if (r < rows && k < K) v = p.kfast ? S[(long long)r * p.ld + k] : S[(long long)k * p.ld + r];
+    if (r < rows && k < K) {
+      const int row = p.gather ? p.gather[r] : r;
+      if (row >= 0) v = p.kfast ? S[(long long)row * p.ld + k] : S[(long long)k * p.ld + row];
+    }
     if (p.conj) v.y = -v.y;
     if (p.kfast) tile[t][tx] = v; else tile[tx][t] = v;
   }
@@ -516,6 +524,31 @@ int sm_count() {
   return n > 0 ? n : 148;
 }
 
+// split-K for grids of a few waves: one CTA per SM is resident (the ring
+// takes 192 KB of shared memory), so a grid of T tiles split s ways runs
+// ceil(T s / SMs) waves of K / s blocks each; take the s (<= 32, >= 4 K
+// blocks per split) with the fewest wave-blocks, preferring the smaller s
+// within 3% (each split adds a partial product to write and sum)
+int choose_split(long long tiles, int ktiles) {
+  int split = 1;
+  const long long sms = sm_count();
+  if (tiles < 4 * sms && ktiles >= 8) {
+    double best = 1e300;
+    const int smax = std::min(32, ktiles / 4);
+    for (int sp = 1; sp <= smax; ++sp) {
+      const long long waves = (tiles * sp + sms - 1) / sms;
+      const double cost = (double)waves * (double)((ktiles + sp - 1) / sp);
+      if (cost < 0.97 * best) { best = cost; split = sp; }
+    }
+  }
+  return split;
+}
+
+int k_blocks(int K, int esz) {
+  const int align = 16 / esz, kp = ((2 * K + align - 1) / align) * align;
+  return (kp + (TC_ROW_BYTES / esz) - 1) / (TC_ROW_BYTES / esz);
+}
+
 template <int ESZ>
 cudaError_t run_tc(const GemmArgs& g, TcWork& w, int* err_dev, cudaStream_t st, int* launches) {
   const int esz = ESZ;
@@ -527,7 +560,8 @@ cudaError_t run_tc(const GemmArgs& g, TcWork& w, int* err_dev, cudaStream_t st, 
   const long long instA = (long long)a1 * a2, instB = (long long)bb1 * bb2;
   if (instA > 65535 || instB > 65535) return cudaErrorInvalidValue;
   const size_t a_bytes = (size_t)instA * g.M * kp * esz;
-  const size_t b_bytes = (size_t)instB * 2 * g.N * kp * esz;
+  const int nb = g.group_tile ? 2 * g.N : g.N;   // columns of B
+  const size_t b_bytes = (size_t)instB * 2 * nb * kp * esz;
   cudaError_t e;
   if ((e = w.ensure(0, a_bytes)) != cudaSuccess) return e;
   if ((e = w.ensure(1, a_bytes)) != cudaSuccess) return e;
@@ -546,8 +580,9 @@ cudaError_t run_tc(const GemmArgs& g, TcWork& w, int* err_dev, cudaStream_t st, 
       p.hi = hi; p.lo = lo;
       return p;
     };
-    const PackSide pa = side(g.A, g.lda, g.sA1, g.sA2, g.opA, g.opA == OP_N || g.opA == OP_R, g.M, 0, a2, instA, w.buf[0], w.buf[1]);
-    const PackSide pb = side(g.B, g.ldb, g.sB1, g.sB2, g.opB, g.opB == OP_T || g.opB == OP_C, g.N, 1, bb2, instB, w.buf[2], w.buf[3]);
+    PackSide pa = side(g.A, g.lda, g.sA1, g.sA2, g.opA, g.opA == OP_N || g.opA == OP_R, g.M, 0, a2, instA, w.buf[0], w.buf[1]);
+    const PackSide pb = side(g.B, g.ldb, g.sB1, g.sB2, g.opB, g.opB == OP_T || g.opB == OP_C, nb, 1, bb2, instB, w.buf[2], w.buf[3]);
+    pa.gather = g.a_rows;
     const long long blocks = (long long)gx * (pa.gy * instA + pb.gy * instB);
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     pack_kernel<ESZ><<<(unsigned)blocks, 256, 0, st>>>(pa, pb, g.K, kp, gx);
@@ -556,8 +591,8 @@ cudaError_t run_tc(const GemmArgs& g, TcWork& w, int* err_dev, cudaStream_t st, 
   CUtensorMap tAh, tAl, tBh, tBl;
   if (!make_map(&tAh, esz, w.buf[0], kp, g.M, (int)instA, TC_BM) ||
       !make_map(&tAl, esz, w.buf[1], kp, g.M, (int)instA, TC_BM) ||
-      !make_map(&tBh, esz, w.buf[2], kp, 2 * g.N, (int)instB, TC_BN) ||
-      !make_map(&tBl, esz, w.buf[3], kp, 2 * g.N, (int)instB, TC_BN))
+      !make_map(&tBh, esz, w.buf[2], kp, 2 * nb, (int)instB, TC_BN) ||
+      !make_map(&tBl, esz, w.buf[3], kp, 2 * nb, (int)instB, TC_BN))
     return cudaErrorInvalidValue;
   TcArgs a{};
   a.M = g.M; a.N = g.N;
@@ -574,22 +609,9 @@ cudaError_t run_tc(const GemmArgs& g, TcWork& w, int* err_dev, cudaStream_t st, 
     const long long tm = (g.M + TC_BM - 1) / TC_BM;
     tiles = tm * (tm + 1) / 2;
   }
-  // split-K for grids of a few waves: one CTA per SM is resident (the ring
-  // takes 192 KB of shared memory), so a grid of T tiles split s ways runs
-  // ceil(T s / SMs) waves of K / s blocks each; take the s (<= 32, >= 4 K
-  // blocks per split) with the fewest wave-blocks, preferring the smaller s
-  // within 3% (each split adds a partial product to write and sum)
-  int split = 1;
-  const long long sms = sm_count();
-  if (tiles < 4 * sms && a.ktiles >= 8) {
-    double best = 1e300;
-    const int smax = std::min(32, a.ktiles / 4);
-    for (int sp = 1; sp <= smax; ++sp) {
-      const long long waves = (tiles * sp + sms - 1) / sms;
-      const double cost = (double)waves * (double)((a.ktiles + sp - 1) / sp);
-      if (cost < 0.97 * best) { best = cost; split = sp; }
-    }
-  }
+  int split = g.split > 0 ? std::min(g.split, a.ktiles) : choose_split(tiles, a.ktiles);
+  a.grp = g.group_tile;
+  a.grp_row = 2 * g.N;
   if ((long long)g.b1 * g.b2 * split > 65535) split = 1;
   a.per = (a.ktiles + split - 1) / split;
   split = (a.ktiles + a.per - 1) / a.per;   // every split owns at least one K block
@@ -648,6 +670,11 @@ void TcWork::release() {
     buf[i] = nullptr;
     cap[i] = 0;
   }
+}
+
+int gemm_tc_split(int M, int N, int K, int precision) {
+  const long long tiles = (long long)((2 * N + TC_BN - 1) / TC_BN) * ((M + TC_BM - 1) / TC_BM);
+  return choose_split(tiles, k_blocks(K, precision == DMRGC_BF16X3 ? 2 : 4));
 }
 
 cudaError_t gemm_tc(const GemmArgs& g, int precision, TcWork& w, int* err_dev, cudaStream_t st, int* launches) {

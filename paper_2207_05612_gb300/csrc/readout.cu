@@ -120,6 +120,53 @@ __global__ void ones_kernel(C2* __restrict__ V, int B) {
   if (b < B) V[b] = C2{1, 0};
 }
 
+// One CTA per site: stable partition of the strings by their bit (common.cuh,
+// group_rows).  1024 threads take consecutive runs of strings.
+__global__ void __launch_bounds__(1024) group_rows_kernel(const unsigned char* __restrict__ bits, int B, int n,
+                                                          const int* __restrict__ order, int M, int* __restrict__ pos,
+                                                          int* __restrict__ src, int* __restrict__ tile) {
+  __shared__ int wsum[32];
+  __shared__ int s_zeros;
+  const int i = blockIdx.x, q = order[i], tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  for (int p = tid; p < M; p += 1024) src[(size_t)i * M + p] = -1;
+  const int per = (B + 1023) / 1024, lo = min(B, tid * per), hi = min(B, lo + per);
+  int zeros = 0;
+  for (int b = lo; b < hi; ++b) zeros += (bits[(size_t)b * n + q] & 1) == 0;
+  int incl = zeros;   // zeros before this thread's run: scan over the warp, then the warps
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) wsum[w] = incl;
+  __syncthreads();
+  int before = incl - zeros;
+  for (int k = 0; k < w; ++k) before += wsum[k];
+  if (tid == 1023) s_zeros = before + zeros;
+  __syncthreads();
+  const int start1 = (s_zeros + 127) / 128 * 128;
+  if (tid == 0) tile[i] = start1 / 128;
+  int z = before, o = lo - before;
+  for (int b = lo; b < hi; ++b)
+    pos[(size_t)i * B + b] = (bits[(size_t)b * n + q] & 1) == 0 ? z++ : start1 + o++;
+}
+
+// src[i][pos[i][b]] = pos[i - 1][b]
+__global__ void group_source_kernel(const int* __restrict__ pos, int B, int M, int* __restrict__ src) {
+  const int i = blockIdx.y;
+  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < B; b += gridDim.x * blockDim.x)
+    src[(size_t)i * M + pos[(size_t)i * B + b]] = i > 0 ? pos[(size_t)(i - 1) * B + b] : 0;
+}
+
+__global__ void amp_store_rows_kernel(const float2* __restrict__ V, const int* __restrict__ pos, int B,
+                                      double2* __restrict__ out) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b < B) {
+    const float2 v = V[pos[b]];
+    out[b] = double2{(double)v.x, (double)v.y};
+  }
+}
+
 // Metropolis chains (App. C): counters g (n + 1) + q (bit q, qubit order,
 // 1 iff u >= 1/2) and g (n + 1) + n (acceptance), g = chain (steps + 1) + t.
 __global__ void metro_draw_kernel(unsigned char* __restrict__ prop, double* __restrict__ uacc, int C, int n,
@@ -191,6 +238,20 @@ cudaError_t sample_select(const void* W, const void* T, int B, int r, unsigned l
     sample_select_kernel<<<B, threads, 0, st>>>(reinterpret_cast<const float2*>(W),
                                                 reinterpret_cast<const float2*>(T), r, seed, row0, n, site, qubit,
                                                 out, reinterpret_cast<float2*>(V));
+  return cudaGetLastError();
+}
+
+cudaError_t group_rows(const unsigned char* bits, int B, int n, const int* order, int M, int* pos, int* src, int* tile,
+                       cudaStream_t st) {
+  group_rows_kernel<<<n, 1024, 0, st>>>(bits, B, n, order, M, pos, src, tile);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  group_source_kernel<<<dim3((unsigned)std::min(64, (B + 255) / 256), (unsigned)n), 256, 0, st>>>(pos, B, M, src);
+  return cudaGetLastError();
+}
+
+cudaError_t amp_store_rows(const void* V, const int* pos, int B, double2* out, cudaStream_t st) {
+  amp_store_rows_kernel<<<(B + 255) / 256, 256, 0, st>>>(reinterpret_cast<const float2*>(V), pos, B, out);
   return cudaGetLastError();
 }
 

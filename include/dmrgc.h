@@ -101,16 +101,20 @@ typedef struct {
                                  sweep cutoff); 0 (default): the bond is the product of the
                                  straddling gates' Schmidt ranks */
   int svd_path;               /* complex64 modes, truncated SVDs of 128..2048 rows that keep
-                                 fewer than all of them (the sweep's theta, the zip-up's Gram):
+                                 fewer than all of them (the sweep's theta, the zip-up's Gram)
+                                 and, in the sweep, of more than 192 rows that may keep all:
                                  0 (default) = the leading eigenvectors of the Gram matrix
                                  G G^+ (TF32x3 product, Householder tridiagonalisation,
                                  bisection and FP64 inverse iteration, back-transformation)
                                  whenever every kept eigenvalue is at least 1e-5 of the largest
                                  (the Gram's rounding then cannot move the kept subspace) and a
-                                 count set by the cutoff has cutoff^2 at or above that level,
-                                 the Jacobi SVD otherwise or when the eigensolver meets a
-                                 non-finite value; 1 = always the Jacobi SVD.  FP64 mode
-                                 always uses the Jacobi SVD. */
+                                 count set by the cutoff has cutoff^2 at or above that level;
+                                 in the sweep (svd_mode 0, no rank records) a spectrum that
+                                 reaches lower is taken in up to four parts, each from the Gram
+                                 matrix of what the earlier ones leave of theta; the Jacobi SVD
+                                 otherwise or when the eigensolver meets a non-finite value;
+                                 1 = always the Jacobi SVD.  FP64 mode always uses the Jacobi
+                                 SVD. */
 } dmrgc_options;
 
 typedef struct {
@@ -328,21 +332,22 @@ dmrgc_status dmrgc_test_svd(int precision, int m, int n, const double* G, int ch
  * only (1..3); 3 <= m <= 2048; 1 <= chi < m.  s_out[m]: the min(chi+1, m)
  * leading singular values, zeros after; U_out[m][k] row-major.  *k_out = k,
  * or -1 when the kept eigenvalues are not all resolved (lambda_{k-1} < 1e-5
- * lambda_0, or rel_cut set k while rel_cut^2 < 1e-5): the sweep then uses the
- * Jacobi SVD. */
+ * lambda_0, or rel_cut set k while rel_cut^2 < 1e-5): the sweep then takes the
+ * spectrum in parts or uses the Jacobi SVD (options.svd_path). */
 dmrgc_status dmrgc_test_svd_gram(int precision, int m, int n, const double* G, int chi, double rel_cut,
                                  double* s_out, int* k_out, double* U_out);
 
 /* Tuning: the Jacobi kernel for complex64 matrices of at most 1024 rows
- * (process-wide).  0 (default): column pairs, one warp per column, two
- * 4-column blocks per CTA; 1: 8 x 8 Gram blocks, rows spread over 512 threads,
+ * (process-wide).  0 (default): column pairs, one warp per column; the whole
+ * matrix in one thread-block cluster up to 512 rows and 256 columns (128 above
+ * 256 rows), two 4-column blocks per CTA of a grid beyond; 1: 8 x 8 Gram blocks, rows spread over 512 threads,
  * one Jacobi sweep of the Gram per round.  Both compute the same
  * decomposition to working precision.  Other values: DMRGC_EINVAL. */
 dmrgc_status dmrgc_set_jacobi_kernel(int variant);
 
 /* Failure handling: the iteration limit of every spin wait of the Jacobi
- * kernels on the current device (the bounded grid barrier and the per-block
- * round counters; one poll is about 64 ns).  A wait that runs out sets the
+ * kernels on the current device (the bounded grid barrier, the per-block round
+ * counters and the cluster kernels' mbarriers; one poll is about 64 ns).  A wait that runs out sets the
  * launch's error flag, every CTA leaves at its next wait, and the calling
  * entry point returns DMRGC_ETIMEOUT; the context stays usable.  0 restores
  * the default (2e7 polls, about 1.3 s).  Process-wide per device. */

@@ -6,9 +6,11 @@
 // theta^+ for the right ones), formed by the contraction engine.  This file
 // diagonalises H in three steps instead of the one-sided Jacobi sweeps:
 //
-//  1. he_tridiag_kernel: unitary Householder reduction H = Q T Q^+ with T
+//  1. he_tridiag_kernel and, for the last 512 rows, he_tridiag_cluster_kernel
+//     (one thread-block cluster, the exchange through distributed shared
+//     memory): unitary Householder reduction H = Q T Q^+ with T
 //     real symmetric tridiagonal (Q = P_0 P_1 ... P_{n-2}, P_j = I - tau_j u_j u_j^+).
-//     One persistent cooperative kernel; rows are owned by CTAs cyclically and
+//     The first is one persistent cooperative kernel; rows are owned by CTAs cyclically and
 //     kept in shared memory where they fit.  Step j forms column j of the
 //     current matrix, the reflector, p = tau A u over the owned rows
 //     (applying step j-1's rank-2 update A -= u w^+ + w u^+ in the same pass)
@@ -21,8 +23,8 @@
 //  2. tri_bisect_kernel, tri_invit_kernel, tri_cluster_kernel: the leading
 //     eigenvalues of T by Sturm-count multisection (FP32, one warp per
 //     eigenvalue); their eigenvectors by inverse iteration in FP64 (the small
-//     core), one thread per eigenvalue, then modified Gram-Schmidt inside
-//     clusters of close eigenvalues and the Rayleigh quotients.
+//     core), one thread per eigenvalue, then Gram-Schmidt (classical, twice)
+//     inside clusters of close eigenvalues and the Rayleigh quotients.
 //  3. bt_wy_kernel and he_backtrans_kernel: eigenvector of H = Q z.  The
 //     reflectors are grouped in blocks of WY in compact WY form
 //     P_a .. P_{a+WY-1} = I - V Tb V^+ (Tb upper triangular), and each block is
@@ -31,10 +33,11 @@
 // H is scaled by 1/max_i H_ii first, so every entry lies in [-1, 1] whatever
 // the scale of theta.  The Gram squares the condition number: eigenvalues
 // carry an absolute error of about eps |H|, so singular values below ~1e-3
-// s_1 are not resolved.  The caller therefore uses this path only when the
+// s_1 are not resolved.  The caller therefore takes a result only when the
 // kept eigenvalues all lie well above that level (lambda_{k-1} >= 1e-5
-// lambda_0, set by the caller); otherwise, or when the eigensolver meets a
-// non-finite value, the update falls back to the Jacobi SVD of theta itself.
+// lambda_0, set by the caller); a spectrum that reaches lower it takes in
+// parts, from the Gram matrices of the residuals, or, as when the eigensolver
+// meets a non-finite value, by the Jacobi SVD of theta itself.
 #include <cooperative_groups.h>
 
 #include <algorithm>

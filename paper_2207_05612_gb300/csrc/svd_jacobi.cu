@@ -4,9 +4,12 @@
 // for a pair (u, v) with alpha = |u|^2, beta = |v|^2, gamma = u^+ v, a unitary
 // 2x2 rotation zeroes gamma.  Pairs follow the round-robin (circle) order, so
 // one round holds n/2 disjoint pairs that run in parallel, one warp per pair;
-// n-1 rounds make a sweep.  All sweeps run in one persistent cooperative
-// kernel: rounds are separated by a grid barrier whose wait is bounded (an
-// exhausted wait sets an error flag and every CTA returns).  Convergence: a
+// n-1 rounds make a sweep.  All sweeps run in one persistent kernel: a matrix
+// that fits one thread-block cluster stays in its registers and moves through
+// distributed shared memory; a larger one is worked on by a cooperative grid
+// whose rounds are separated by a grid barrier.  Every wait is bounded (an
+// exhausted one sets an error flag and every CTA returns).  A wide matrix is
+// reduced to its square L factor first where one cluster holds it.  Convergence: a
 // sweep whose largest |gamma|/sqrt(alpha beta) is below tol ends the loop.
 //
 // On return the columns of W = G V are mutually orthogonal; their norms are

@@ -232,6 +232,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  chain_enter();   // barriers and TMEM were set up while the pack was running
 
   if (warp == 0 && lane == 0) {
     // ---- TMA producer
@@ -408,6 +409,7 @@ struct PackSide {
 template <int ESZ>
 __global__ void __launch_bounds__(256) pack_kernel(PackSide A, PackSide B, int K, int kp, int gx) {
   __shared__ float2 tile[32][33];
+  chain_enter();
   const bool second = blockIdx.x >= A.blocks;
   const PackSide& p = second ? B : A;
   unsigned id = second ? blockIdx.x - A.blocks : blockIdx.x;
@@ -467,6 +469,7 @@ __global__ void __launch_bounds__(256) pack_kernel(PackSide A, PackSide B, int K
 // the same bit for bit from run to run: C (+)= sum_s P[s][batch]
 __global__ void splitk_reduce_kernel(const float2* __restrict__ P, int split, int nbatch, float2* C, int M, int N,
                                      long long ldc, long long s1, long long s2, int b2, int beta_one) {
+  chain_enter();
   const int batch = blockIdx.z;
   float2* Cb = C + (long long)(batch / b2) * s1 + (long long)(batch % b2) * s2;
   const long long mn = (long long)M * N;
@@ -585,8 +588,8 @@ cudaError_t run_tc(const GemmArgs& g, TcWork& w, int* err_dev, cudaStream_t st, 
     pa.gather = g.a_rows;
     const long long blocks = (long long)gx * (pa.gy * instA + pb.gy * instB);
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    pack_kernel<ESZ><<<(unsigned)blocks, 256, 0, st>>>(pa, pb, g.K, kp, gx);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_chained(pack_kernel<ESZ>, dim3((unsigned)blocks), dim3(256), 0, st, pa, pb, g.K, kp, gx)) != cudaSuccess)
+      return e;
   }
   CUtensorMap tAh, tAl, tBh, tBl;
   if (!make_map(&tAh, esz, w.buf[0], kp, g.M, (int)instA, TC_BM) ||
@@ -630,15 +633,15 @@ cudaError_t run_tc(const GemmArgs& g, TcWork& w, int* err_dev, cudaStream_t st, 
   a.total = (upper ? (long long)a.tiles_m * (a.tiles_m + 1) / 2 : (long long)a.tiles_n * a.tiles_m) *
             nbatch * split;
   const long long ctas = std::min<long long>(a.total, (long long)sm_count());
-  tc_gemm_kernel<ESZ><<<(unsigned)ctas, TC_THREADS, TC_SMEM_BYTES, st>>>(tAh, tAl, tBh, tBl, a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = launch_chained(tc_gemm_kernel<ESZ>, dim3((unsigned)ctas), dim3(TC_THREADS), TC_SMEM_BYTES, st, tAh, tAl, tBh, tBl,
+                          a)) != cudaSuccess)
+    return e;
   if (split > 1) {
     const long long mn = (long long)g.M * g.N;
     int bx = (int)std::min<long long>((mn + 255) / 256, 1024);
     dim3 rg(bx < 1 ? 1 : bx, 1, (unsigned)nbatch);
-    splitk_reduce_kernel<<<rg, 256, 0, st>>>(a.P, split, nbatch, (float2*)g.C, g.M, g.N, g.ldc, g.sC1, g.sC2, g.b2,
-                                             g.beta_one);
-    e = cudaGetLastError();
+    e = launch_chained(splitk_reduce_kernel, rg, dim3(256), 0, st, a.P, split, nbatch, (float2*)g.C, g.M, g.N, g.ldc,
+                       g.sC1, g.sC2, g.b2, g.beta_one);
   }
   return e;
 }

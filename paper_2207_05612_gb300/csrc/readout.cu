@@ -33,6 +33,7 @@ __device__ __forceinline__ double splitmix64_uniform(unsigned long long seed, un
 template <typename C2>
 __global__ void amp_select_kernel(const C2* __restrict__ W, int r, const unsigned char* __restrict__ bits,
                                   int n, const int* __restrict__ qubits, int g, C2* __restrict__ V) {
+  chain_enter();
   const int b = blockIdx.x;
   int x = 0;   // the tensor's physical index: its g qubits, the first the most significant bit
   for (int j = 0; j < g; ++j) x = (x << 1) | (bits[(long long)b * n + qubits[j]] & 1);
@@ -56,6 +57,7 @@ __global__ void sample_select_kernel(const C2* __restrict__ W, const C2* __restr
   __shared__ double red[32];
   __shared__ int s_x;
   __shared__ double s_inv;
+  chain_enter();
   const int b = blockIdx.x;
   const C2* w = W + (long long)b * 2 * r;
   const C2* t = T ? T + (long long)b * 2 * r : nullptr;
@@ -219,26 +221,22 @@ cudaError_t amp_select(const void* W, int B, int r, const unsigned char* bits, i
                        void* V, bool fp64, cudaStream_t st) {
   const int threads = r >= 256 ? 256 : (r >= 64 ? 64 : 32);
   if (fp64)
-    amp_select_kernel<<<B, threads, 0, st>>>(reinterpret_cast<const double2*>(W), r, bits, n, qubits, g,
-                                             reinterpret_cast<double2*>(V));
-  else
-    amp_select_kernel<<<B, threads, 0, st>>>(reinterpret_cast<const float2*>(W), r, bits, n, qubits, g,
-                                             reinterpret_cast<float2*>(V));
-  return cudaGetLastError();
+    return launch_chained(amp_select_kernel<double2>, dim3(B), dim3(threads), 0, st, reinterpret_cast<const double2*>(W), r,
+                          bits, n, qubits, g, reinterpret_cast<double2*>(V));
+  return launch_chained(amp_select_kernel<float2>, dim3(B), dim3(threads), 0, st, reinterpret_cast<const float2*>(W), r,
+                        bits, n, qubits, g, reinterpret_cast<float2*>(V));
 }
 
 cudaError_t sample_select(const void* W, const void* T, int B, int r, unsigned long long seed, long long row0, int n,
                           int site, int qubit, unsigned char* out, void* V, bool fp64, cudaStream_t st) {
   const int threads = r >= 256 ? 256 : (r >= 64 ? 64 : 32);
   if (fp64)
-    sample_select_kernel<<<B, threads, 0, st>>>(reinterpret_cast<const double2*>(W),
-                                                reinterpret_cast<const double2*>(T), r, seed, row0, n, site, qubit,
-                                                out, reinterpret_cast<double2*>(V));
-  else
-    sample_select_kernel<<<B, threads, 0, st>>>(reinterpret_cast<const float2*>(W),
-                                                reinterpret_cast<const float2*>(T), r, seed, row0, n, site, qubit,
-                                                out, reinterpret_cast<float2*>(V));
-  return cudaGetLastError();
+    return launch_chained(sample_select_kernel<double2>, dim3(B), dim3(threads), 0, st, reinterpret_cast<const double2*>(W),
+                          reinterpret_cast<const double2*>(T), r, seed, row0, n, site, qubit, out,
+                          reinterpret_cast<double2*>(V));
+  return launch_chained(sample_select_kernel<float2>, dim3(B), dim3(threads), 0, st, reinterpret_cast<const float2*>(W),
+                        reinterpret_cast<const float2*>(T), r, seed, row0, n, site, qubit, out,
+                        reinterpret_cast<float2*>(V));
 }
 
 cudaError_t group_rows(const unsigned char* bits, int B, int n, const int* order, int M, int* pos, int* src, int* tile,

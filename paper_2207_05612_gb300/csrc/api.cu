@@ -357,18 +357,24 @@ dmrgc_status eig_try(dmrgc_ctx* c, int bond, const void* G, int rows, int kdim, 
     return DMRGC_OK;
   };
   auto flops = [&](int kept) { c->stats.svd_flops += 16.0 / 3.0 * (double)rows * rows * rows + 8.0 * (double)rows * rows * kept; };
-  // diagonalise what eig_gram left in jw; 1: a size or launch shape the eigensolver does not take
+  // a size or launch shape the eigensolver does not take, as against an error of the call
+  auto not_taken = [](cudaError_t e) {
+    if (e != cudaErrorInvalidConfiguration && e != cudaErrorInvalidValue) return false;
+    cudaGetLastError();
+    return true;
+  };
+  // diagonalise what eig_gram left in jw.  The error is returned: eig_reduce has
+  // already read and cleared that of a failed launch.
   std::vector<float> lam;
   EigHead head{};
-  auto reduce = [&](int kk) -> int {
+  auto reduce = [&](int kk) {
     Span sp(c, TC_SVD);
     cudaError_t e = eig_reduce(c->jw.p, rows, kk, c->ework.p, c->st, &launches);
-    if (e == cudaErrorInvalidConfiguration || e == cudaErrorInvalidValue) { cudaGetLastError(); return 1; }
     if (e == cudaSuccess && staged) {
       lam.resize(kk);
       e = eig_spectrum(c->ework.p, rows, kk, lam.data(), &head, c->st);
     }
-    return e == cudaSuccess ? 0 : 2;
+    return e;
   };
   TruncResult tr{};
   auto select = [&](int kk, int most, double cut_s, double tie_s, DevBuf& dst, int layout) -> dmrgc_status {
@@ -376,7 +382,7 @@ dmrgc_status eig_try(dmrgc_ctx* c, int bond, const void* G, int rows, int kdim, 
       Span sp(c, TC_SVD);
       const cudaError_t e = eig_select(c->jw.p, rows, kk, most, cut_s, tie_s, kEigResolve, c->ework.p, c->tres.p, dst.p,
                                        layout, c->st, &launches);
-      if (e == cudaErrorInvalidConfiguration || e == cudaErrorInvalidValue) { cudaGetLastError(); tr.status = 1; return DMRGC_OK; }
+      if (not_taken(e)) { tr.status = 1; return DMRGC_OK; }
       CK(e);
     }
     CK(cudaMemcpyAsync(&tr, c->tres.p, sizeof(tr), cudaMemcpyDeviceToHost, c->st));
@@ -388,9 +394,9 @@ dmrgc_status eig_try(dmrgc_ctx* c, int bond, const void* G, int rows, int kdim, 
 
   TRY(eig_gram(c, G, rows, kdim, conj_cols, gp));
   int kk = std::min(c->chi + 1, rows);
-  int rc = reduce(kk);
-  if (rc == 1) return declined();
-  CK(rc == 0 ? cudaSuccess : cudaGetLastError());
+  cudaError_t reduced = reduce(kk);
+  if (not_taken(reduced)) return declined();
+  CK(reduced);
   auto direct = [&]() -> dmrgc_status {   // one stage, straight into the caller's layout
     TRY(select(kk, kmax, cut, tie, out, mode));
     c->last_tr = tr;
@@ -449,9 +455,9 @@ dmrgc_status eig_try(dmrgc_ctx* c, int bond, const void* G, int rows, int kdim, 
     if (rows <= 256) return declined();
     TRY(eig_gram(c, cur, rows, kdim, conj_cols, gp));
     kk = std::min(kmax - total + 1, rows);
-    rc = reduce(kk);
-    if (rc == 1) return declined();
-    CK(rc == 0 ? cudaSuccess : cudaGetLastError());
+    reduced = reduce(kk);
+    if (not_taken(reduced)) return declined();
+    CK(reduced);
     if (head.err) return fail(c, DMRGC_ETIMEOUT, "Gram eigensolver wait timed out");
     if (!std::isfinite(lam[0])) return declined();
     if (!((double)lam[0] * head.unit > cutabs)) finished = true;

@@ -258,31 +258,37 @@ constexpr int kEigMinN = 128, kEigStages = 4;
 // What the eigensolver takes.  Where rows are dropped (chi < rows): from 128 rows
 // on.  In the sweep also matrices of which every row may be kept, from 193 rows
 // on (the cluster Jacobi kernel takes 0.9 ms at 128 x 128 and 2.7 ms at 256 x 256,
-// the eigensolver with all vectors 0.7 and 1.6 ms), but not tall ones of at most
-// 256 columns, where the Jacobi kernels work on the short side.
+// the eigensolver with all vectors 0.7 and 1.6 ms).  But not tall thetas of at most
+// 256 columns, where the Jacobi kernels work on the short side: with every row
+// kept any, else those of four rows a column (host copies included, 1024 x 256: 6 to
+// 10 ms against 9 to 23 ms, 512 x 128: 2 to 3 against 3 to 7, 512 x 256: even).
 bool eig_applies(const dmrgc_ctx* c, int rows, int kdim, bool sweep) {
   if (c->fp64 || c->opt.svd_path != 0 || rows < kEigMinN || rows > 2048) return false;
-  if (c->chi < rows) return true;
-  return sweep && rows > 192 && !(kdim < rows && kdim <= 256);
+  const bool drops = c->chi < rows;
+  if (sweep && kdim <= 256 && (drops ? 4 * kdim <= rows : kdim < rows)) return false;
+  return drops || (sweep && rows > 192);
 }
 
-// The staged form: where the spectrum itself is not recorded, above 256 rows, and
-// below that where rows need not be dropped: the usual case there is a matrix of
+// The form it takes a matrix in, by what it resolves.  0: it does not take it;
+// 1: one Gram matrix; 2: one, and the residual if that is noise; 3: stages.
+// Stages run where the spectrum itself is not recorded, above 256 rows, and below that,
+// as form 2, where rows need not be dropped: the usual case there is a matrix of
 // lower rank, which ends with the first residual (a second diagonalisation
 // would be slower than the cluster Jacobi kernel: eig_try declines).
-bool eig_staged(const dmrgc_ctx* c, int rows, bool sweep) {
-  return sweep && (rows > 256 || c->chi >= rows) && c->opt.svd_mode == 0 && !c->opt.log_rank_records;
+int eig_form(const dmrgc_ctx* c, int rows, int kdim, bool sweep) {
+  if (!eig_applies(c, rows, kdim, sweep)) return 0;
+  if (!sweep || (rows <= 256 && c->chi < rows) || c->opt.svd_mode != 0 || c->opt.log_rank_records) return 1;
+  return rows > 256 ? 3 : 2;
 }
 
-// After a truncated SVD at `bond` (either path): should its next one in this
-// layer try the eigensolver?  Spectra change little between visits of a bond, so
-// a matrix it declined (a cluster too long, or stages that did not end) goes
-// straight to the Jacobi SVD; in the modes without stages the spectrum decides,
-// whichever path found it.
-void note_resolvable(dmrgc_ctx* c, int bond, bool eig) {
-  if (bond < 0 || bond >= (int)c->eig_ok.size()) return;
-  const bool plain = c->opt.svd_mode == 0 && !c->opt.log_rank_records;
-  c->eig_ok[bond] = (plain ? eig : !c->last_tr.by_cut && c->last_tr.tail >= kEigResolve) ? 1 : 0;
+// After a truncated SVD at `bond` in the modes without stages: the spectrum decides,
+// whichever path found it, whether the bond's next SVD in this layer tries the
+// eigensolver.  Spectra change little between visits of a bond.  (With stages
+// eig_try notes what it declined.)
+void note_resolvable(dmrgc_ctx* c, int bond) {
+  if (bond < 0 || bond >= (int)c->eig_declined.size()) return;
+  if (c->opt.svd_mode == 0 && !c->opt.log_rank_records) return;
+  c->eig_declined[bond] = (!c->last_tr.by_cut && c->last_tr.tail >= kEigResolve) ? 0 : 1;
 }
 
 // H = G G^+ into c->jw (upper tiles only: the eigensolver mirrors them)
@@ -334,9 +340,14 @@ dmrgc_status eig_project(dmrgc_ctx* c, void* R, int rows, int kdim, bool conj_co
 dmrgc_status eig_try(dmrgc_ctx* c, int bond, const void* G, int rows, int kdim, bool conj_cols, double cut,
                      double tie, DevBuf& out, int mode, int& k, bool& done, bool sweep = false) {
   done = false;
-  if (!eig_applies(c, rows, kdim, sweep)) return DMRGC_OK;
-  const bool staged = eig_staged(c, rows, sweep);
-  if (bond >= 0 && bond < (int)c->eig_ok.size() && !c->eig_ok[bond]) {
+  const int form = eig_form(c, rows, kdim, sweep);
+  if (form == 0) return DMRGC_OK;   // says nothing of the bond's other matrices
+  const bool staged = form > 1, noted = bond >= 0 && bond < (int)c->eig_declined.size();
+  // a spectrum that this form or a more capable one declined at this bond (a
+  // cluster too long, or stages that did not end) goes straight to the Jacobi SVD
+  // until the next layer: it changes little between visits and is the same in both
+  // directions
+  if (noted && form <= c->eig_declined[bond]) {
     c->stats.eig_skipped++;
     return DMRGC_OK;
   }
@@ -353,6 +364,7 @@ dmrgc_status eig_try(dmrgc_ctx* c, int bond, const void* G, int rows, int kdim, 
   };
   auto declined = [&] {   // the Jacobi SVD decides
     c->stats.eig_fallbacks++;
+    if (noted && sweep) c->eig_declined[bond] = (char)form;
     count();
     return DMRGC_OK;
   };
@@ -766,7 +778,7 @@ dmrgc_status update_ltr(dmrgc_ctx* c, int i) {
       CK(gather_columns(c->jw.p, mrow, c->svd_n, k, c->tres.p, false, 0, c->A[i].p, c->fp64, c->st));
       c->stats.kernel_launches++;
     }
-    note_resolvable(c, i, eig);
+    note_resolvable(c, i);
     TRY(record_end(c, i, k, true, rec));
   }
   TRY(ensure(c, c->A[i + 1], (size_t)k * ncol * c->esz));
@@ -835,7 +847,7 @@ dmrgc_status update_rtl(dmrgc_ctx* c, int i) {
       CK(gather_columns(c->jw.p, ncol, c->svd_n, k, c->tres.p, false, 2, c->A[i + 1].p, c->fp64, c->st));
       c->stats.kernel_launches++;
     }
-    note_resolvable(c, i, eig);
+    note_resolvable(c, i);
     TRY(record_end(c, i, k, true, rec));
   }
   TRY(ensure(c, c->A[i], (size_t)mrow * k * c->esz));
@@ -1327,7 +1339,7 @@ dmrgc_status ctx_setup(dmrgc_ctx* c, int n_qubits, const dmrgc_grid* grid, int c
   c->layer_no = 0;
   c->visit_layer.assign(n_qubits, -1);
   c->kprev.assign(n_qubits, 0);
-  c->eig_ok.assign(n_qubits, 1);
+  c->eig_declined.assign(n_qubits, 0);
   c->rs_ctr = 0;
   c->rs_p = c->opt.rsvd_oversample > 0 ? c->opt.rsvd_oversample : 8;
   c->rs_pow = c->opt.rsvd_power_iters >= 0 ? c->opt.rsvd_power_iters : 1;
@@ -1542,7 +1554,7 @@ dmrgc_status dmrgc_apply_layer(dmrgc_ctx* c, const dmrgc_gate* gates, int n_gate
   c->layer_no++;
   // a new layer changes every spectrum: the first visit of each bond tries
   // the eigensolver again
-  std::fill(c->eig_ok.begin(), c->eig_ok.end(), 1);
+  std::fill(c->eig_declined.begin(), c->eig_declined.end(), 0);
   TRY(build_mpo(c, gates, n_gates));
   if (c->ng > 0) {   // single-site variant: random guess in orthogonal form
     TRY(grouped_guess(c));

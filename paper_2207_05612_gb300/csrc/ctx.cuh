@@ -53,7 +53,7 @@ struct dmrgc_ctx {
   DevBuf df_r, df_c, df_u[4];   // its stages: the residual, U^+ residual, the vectors of each stage
   TruncResult last_tr{};          // result of the last truncated SVD (either path)
   int svd_n = 0;                  // columns of the matrix the last Jacobi SVD ended with (svd_columns)
-  std::vector<char> eig_ok;       // per bond: its next SVD in this layer tries the eigensolver (note_resolvable)
+  std::vector<char> eig_declined; // per bond: the eigensolver's most capable form that declined it in this layer (eig_try)
   DevBuf rv[3];    // read-outs: running rows V, site products W = V A_i, T = W E_i
   DevBuf rv_rows;  // rows of the strings at every site (amplitudes on the tensor cores)
   TcWork tcw;

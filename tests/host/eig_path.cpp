@@ -69,7 +69,7 @@ static void setup(dmrgc_ctx& c, int chi, int bonds) {
   c.sweep_cut = 2e-5;
   c.zero_rel = 1e-5;
   c.tie_rel = 1e-5;
-  c.eig_ok.assign(bonds, 1);
+  c.eig_declined.assign(bonds, 0);
   g_reduces = 0;
   g_fail_at = 0;
   g_status = 0;
@@ -105,8 +105,61 @@ static void failed_reduction() {
       }
 }
 
+// One update at bond 1: prints what became of it.
+static void update(dmrgc_ctx& c, const char* name, int rows, int cols, bool right) {
+  const long long skipped = c.stats.eig_skipped, declined = c.stats.eig_fallbacks;
+  const int reduces = g_reduces;
+  bool done = false;
+  const dmrgc_status s = visit(c, 1, rows, cols, right, done);
+  note_resolvable(&c, 1);
+  const char* what = s != DMRGC_OK ? "error" : done ? "taken" : c.stats.eig_skipped > skipped ? "skipped"
+                     : c.stats.eig_fallbacks > declined ? "declined" : g_reduces > reduces ? "lost" : "not tried";
+  std::printf("%s %d x %d %s: %s\n", name, rows, cols, right ? "right to left" : "left to right", what);
+}
+
+static void visits() {
+  dmrgc_ctx a;
+  setup(a, 600, 4);   // every row may be kept; the residual is noise
+  update(a, "tall then wide", 600, 250, false);
+  update(a, "tall then wide", 600, 250, true);
+  update(a, "tall then wide", 600, 250, false);
+  dmrgc_ctx b;
+  setup(b, 600, 4);
+  g_residual = 1e-3;  // what 250 rows decline, 300 rows take in stages
+  update(b, "grown bond", 250, 400, false);
+  update(b, "grown bond", 250, 400, false);
+  update(b, "grown bond", 300, 400, false);
+  update(b, "grown bond", 250, 400, false);
+  dmrgc_ctx d;
+  setup(d, 200, 4);
+  g_status = 1;       // unresolved by one Gram matrix
+  update(d, "one Gram matrix", 250, 400, false);
+  update(d, "one Gram matrix", 250, 400, false);
+  g_status = 0;
+  update(d, "one Gram matrix", 400, 400, true);
+  dmrgc_ctx e;
+  setup(e, 200, 4);
+  g_status = 1;       // not taken in stages either: nothing takes it
+  update(e, "stages", 400, 400, false);
+  g_status = 0;
+  update(e, "stages", 400, 400, true);
+  update(e, "stages", 250, 400, false);
+  dmrgc_ctx r;
+  setup(r, 200, 4);
+  r.opt.log_rank_records = 1;   // the recorded spectrum decides
+  g_status = 1;
+  r.last_tr.tail = 1.0;
+  update(r, "records", 400, 400, false);
+  g_status = 0;
+  r.last_tr.by_cut = 0;
+  r.last_tr.tail = 1.0;
+  note_resolvable(&r, 1);       // a Jacobi SVD found it resolved
+  update(r, "records", 400, 400, true);
+}
+
 int main(int argc, char** argv) {
   (void)argc;
   if (std::string(argv[1]) == "failed_reduction") failed_reduction();
+  if (std::string(argv[1]) == "visits") visits();
   return 0;
 }

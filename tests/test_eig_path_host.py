@@ -45,3 +45,26 @@ def test_failed_reduction_is_an_error(host):
                 want.append(f"reduce rows={rows} call={call} error={error}: status={0 if error == 9 else 3} done=0 "
                             f"declined={1 if error == 9 else 0}")
     assert got == want
+
+
+def test_bond_visits(host):
+    """Which updates of one bond try the eigensolver.  A matrix that it does not take
+    says nothing of the bond's other direction; a declined spectrum sends to the
+    Jacobi SVD what resolves no more than the form that declined it."""
+    assert host("visits") == [
+        "tall then wide 600 x 250 left to right: not tried",
+        "tall then wide 600 x 250 right to left: taken",
+        "tall then wide 600 x 250 left to right: not tried",
+        "grown bond 250 x 400 left to right: declined",
+        "grown bond 250 x 400 left to right: skipped",
+        "grown bond 300 x 400 left to right: taken",
+        "grown bond 250 x 400 left to right: skipped",
+        "one Gram matrix 250 x 400 left to right: declined",
+        "one Gram matrix 250 x 400 left to right: skipped",
+        "one Gram matrix 400 x 400 right to left: taken",
+        "stages 400 x 400 left to right: declined",
+        "stages 400 x 400 right to left: skipped",
+        "stages 250 x 400 left to right: skipped",
+        "records 400 x 400 left to right: declined",
+        "records 400 x 400 right to left: taken",
+    ]

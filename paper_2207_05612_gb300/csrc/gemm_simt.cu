@@ -235,24 +235,33 @@ int simt_sms() {
   return n > 0 ? n : 148;
 }
 
-// Split of a small-tile product (0: use the 64 x 64 tiles).  Both kernels run at
-// the FMA rate once their SMs are busy, so a product costs its waves of tiles over
-// the SMs times the work of one tile; the split takes the fewest (at least 2 K
-// blocks per CTA, clusters of at most 8 CTAs).
-int small_split(const GemmArgs& g, long long batch) {
-  const long long sms = simt_sms();
+// Split of a small-tile product on `sms` SMs (0: use the 64 x 64 tiles): the fewest
+// waves of tiles over the SMs times the K blocks of one tile (at least 2 K blocks per
+// CTA, clusters of at most 8 CTAs), if that is less than what the 64 x 64 tiles
+// cost in the same unit, with 10% for the larger tile's lower overhead per FMA.
+//
+// FP64: both kernels run at the FMA rate once their SMs are busy, so a large tile
+// costs 16 small ones.
+// FP32: the small kernel issues two shared-memory loads for four FMAs and reaches
+// half of the large one's rate, which in turn needs several CTAs an SM: w waves of
+// large tiles cost 7 + 6 w (fitted to 41 sizes).  1024 x 1024 x 512: 139 us on large
+// tiles, 207 on small ones; 2048 x 1024 x 512: 233 and 406; 512 x 512 x 512: 107 and
+// 62; 64 x 64 x 512: 106 and 8; even at 160 large tiles.  A split has to save a
+// sixteenth here (640 x 1024 x 512: 135 us in one piece, 151 in eight).
+int small_split(const GemmArgs& g, long long batch, bool fp64, long long sms) {
   const long long t64 = (long long)((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN) * batch;
   const long long tm = (g.M + ST - 1) / ST, tn = (g.N + ST - 1) / ST;
   if (tm > 65535 || tn * 8 > INT_MAX) return 0;
   const long long kb = std::max<long long>(1, (g.K + ST - 1) / ST);
-  const long long c64 = (t64 + sms - 1) / sms * (BM * BN / (ST * ST)) * kb;
+  const long long waves = (t64 + sms - 1) / sms;
+  const long long c64 = (fp64 ? waves * (BM * BN / (ST * ST)) : 7 + 6 * waves) * kb;
   long long best = LLONG_MAX;
   int split = 1;
   for (int s = 1; s <= 8 && (s == 1 || kb >= 2 * s); s *= 2) {
     const long long c = (tm * tn * batch * s + sms - 1) / sms * ((kb + s - 1) / s);
-    if (c < best) { best = c; split = s; }
+    if (fp64 || s == 1 ? c < best : 16 * c < 15 * best) { best = c; split = s; }
   }
-  return 10 * best < 9 * c64 ? split : 0;   // the large tile has less overhead per FMA
+  return 10 * best < 9 * c64 ? split : 0;
 }
 
 template <typename R>
@@ -280,7 +289,7 @@ cudaError_t gemm_simt(const GemmArgs& g, bool fp64, cudaStream_t st) {
   if (gy > 65535) return cudaErrorInvalidConfiguration;
   dim3 grid((g.N + BN - 1) / BN, (unsigned)gy, (unsigned)batch);
   // an empty contraction (K <= 0) writes C = 0, or leaves it with beta
-  if (const int S = small_split(g, batch)) return fp64 ? launch_small<double>(g, batch, S, st) : launch_small<float>(g, batch, S, st);
+  if (const int S = small_split(g, batch, fp64, simt_sms())) return fp64 ? launch_small<double>(g, batch, S, st) : launch_small<float>(g, batch, S, st);
   if (fp64)
     gemm_kernel<double, Tile<double>::BK><<<grid, NT, 0, st>>>(g);
   else

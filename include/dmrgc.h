@@ -337,6 +337,16 @@ dmrgc_status dmrgc_test_svd(int precision, int m, int n, const double* G, int ch
 dmrgc_status dmrgc_test_svd_gram(int precision, int m, int n, const double* G, int chi, double rel_cut,
                                  double* s_out, int* k_out, double* U_out);
 
+/* dmrgc_test_svd_theta: the truncated SVD of one update of the sweep, the route
+ * chosen as there: G (m x n, column-major) is theta of a left-to-right update, or
+ * its adjoint of a right-to-left one (right = 1).  *k_out: the kept rank, at most
+ * chi, values above rel_cut (> 0) s_1 and the precision's numerical zero;
+ * U_out[m][k] (row-major, room for min(m, chi) columns): the kept left singular
+ * vectors of G; *parts_out: the Gram matrices they came from, 0 if the Jacobi SVD
+ * gave them (svd_path 1: always), wide matrices reduced to L of G = L Q^+ first. */
+dmrgc_status dmrgc_test_svd_theta(int precision, int svd_path, int right, int m, int n, const double* G, int chi,
+                                  double rel_cut, int* k_out, double* U_out, int* parts_out);
+
 /* Tuning: the Jacobi kernel for complex64 matrices of at most 1024 rows
  * (process-wide).  0 (default): column pairs, one warp per column; the whole
  * matrix in one thread-block cluster up to 512 rows and 256 columns (128 above

@@ -103,6 +103,8 @@ def lib():
                                      C.c_void_p, P(C.c_int), C.c_void_p]
         L.dmrgc_test_svd_gram.argtypes = [C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_int, C.c_double,
                                           C.c_void_p, P(C.c_int), C.c_void_p]
+        L.dmrgc_test_svd_theta.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_int, C.c_double,
+                                           P(C.c_int), C.c_void_p, P(C.c_int)]
         L.dmrgc_svd_noalloc.argtypes = [C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_int, C.c_double,
                                         C.c_void_p, P(C.c_int), C.c_void_p, C.c_void_p]
         L.dmrgc_batch_run.argtypes = [P(BatchItem), C.c_int, C.c_int, P(Options), C.c_void_p, P(C.c_double)]
@@ -121,7 +123,7 @@ def lib():
         L.dmrgc_mlp_loss_grad.argtypes = [fp, fp, fp, C.c_int, P(C.c_float), fp]
         L.dmrgc_mlp_predict.argtypes = [fp, fp, C.c_int, C.c_int, fp]
         for name in ("dmrgc_metropolis", "dmrgc_create_grouped", "dmrgc_group_sizes", "dmrgc_set_mps", "dmrgc_sweep_updates", "dmrgc_set_wait_limit", "dmrgc_xeb", "dmrgc_overlap", "dmrgc_overlap_layer", "dmrgc_set_jacobi_kernel", "dmrgc_set_rank_model", "dmrgc_rank_records", "dmrgc_mlp_train",
-                     "dmrgc_mlp_loss_grad", "dmrgc_mlp_predict", "dmrgc_batch_run", "dmrgc_svd_noalloc", "dmrgc_test_gemm", "dmrgc_test_svd", "dmrgc_test_svd_gram", "dmrgc_default_options", "dmrgc_create", "dmrgc_apply_layer", "dmrgc_sweep",
+                     "dmrgc_mlp_loss_grad", "dmrgc_mlp_predict", "dmrgc_batch_run", "dmrgc_svd_noalloc", "dmrgc_test_gemm", "dmrgc_test_svd", "dmrgc_test_svd_gram", "dmrgc_test_svd_theta", "dmrgc_default_options", "dmrgc_create", "dmrgc_apply_layer", "dmrgc_sweep",
                      "dmrgc_fidelity", "dmrgc_amplitude", "dmrgc_sample", "dmrgc_bond_dims",
                      "dmrgc_get_mps", "dmrgc_step_history", "dmrgc_get_stats", "dmrgc_reset_stats"):
             getattr(L, name).restype = C.c_int
@@ -320,6 +322,19 @@ def dmrgc_test_svd_gram(precision: int, g: np.ndarray, chi: int, rel_cut: float)
     if kk < 0:
         return s, kk, None
     return s, kk, u.reshape(-1)[:m * kk].reshape(m, kk)
+
+
+def dmrgc_test_svd_theta(precision: int, g: np.ndarray, chi: int, rel_cut: float, svd_path: int = 0, right: bool = False):
+    """Truncated SVD of g (m x n) by the route an update of the sweep takes for a
+    theta of this shape, or for its adjoint right to left (diagnostic entry point).
+    Returns (k, U_k, parts): parts = 0 for the Jacobi SVD, else the Gram matrices used."""
+    m, n = g.shape
+    gc = np.asfortranarray(g, dtype=np.complex128)
+    k, parts = C.c_int(), C.c_int()
+    u = np.zeros((m, min(m, chi)), dtype=np.complex128)
+    _check(lib().dmrgc_test_svd_theta(precision, svd_path, int(right), m, n, gc.ctypes.data, chi, rel_cut,
+                                      C.byref(k), u.ctypes.data, C.byref(parts)))
+    return k.value, u.reshape(-1)[:m * k.value].reshape(m, k.value), parts.value
 
 
 def dmrgc_svd_noalloc(precision: int, g_ptr: int, m: int, n: int, chi: int, rel_cut: float,

@@ -340,6 +340,7 @@ dmrgc_status eig_project(dmrgc_ctx* c, void* R, int rows, int kdim, bool conj_co
 dmrgc_status eig_try(dmrgc_ctx* c, int bond, const void* G, int rows, int kdim, bool conj_cols, double cut,
                      double tie, DevBuf& out, int mode, int& k, bool& done, bool sweep = false) {
   done = false;
+  c->eig_parts = 0;
   const int form = eig_form(c, rows, kdim, sweep);
   if (form == 0) return DMRGC_OK;   // says nothing of the bond's other matrices
   const bool staged = form > 1, noted = bond >= 0 && bond < (int)c->eig_declined.size();
@@ -415,6 +416,7 @@ dmrgc_status eig_try(dmrgc_ctx* c, int bond, const void* G, int rows, int kdim, 
     if (tr.status != 0) return declined();   // 1: not resolved, 2: a non-finite value
     k = tr.k;
     done = true;
+    c->eig_parts = 1;
     c->stats.eig_svds++;
     flops(k);
     count();
@@ -484,6 +486,7 @@ dmrgc_status eig_try(dmrgc_ctx* c, int bond, const void* G, int rows, int kdim, 
   }
   k = total;
   done = true;
+  c->eig_parts = parts;
   c->stats.eig_svds++;
   count();
   return DMRGC_OK;
@@ -743,6 +746,29 @@ dmrgc_status record_end(dmrgc_ctx* c, int i, int k, bool full, const std::vector
   return DMRGC_OK;
 }
 
+// Truncated SVD of c->theta (mrow x ncol) as an update takes it: the leading
+// eigenvectors of theta theta^+ (right: theta^+ theta) where they are resolved
+// (eig = true), else the Jacobi SVD.  out: U_k [mrow][k] (right: V_k^+ [k][ncol]).
+dmrgc_status svd_theta(dmrgc_ctx* c, int bond, bool right, int mrow, int ncol, DevBuf& out, int& k, double& f, bool& eig) {
+  const int rows = right ? ncol : mrow, cols = right ? mrow : ncol;
+  TRY(eig_try(c, bond, c->theta.p, rows, cols, right, c->sweep_cut, 0.0, out, right ? 2 : 0, k, eig, true));
+  if (eig) return DMRGC_OK;
+  TRY(ensure(c, c->jw, (size_t)mrow * ncol * c->esz));
+  {
+    // the columns of theta (right: of theta^+, column-major == conj(theta) row-major)
+    Span sp(c, TC_OTHER);
+    CK(right ? copy_conj(c->theta.p, (long long)mrow * ncol, c->jw.p, c->fp64, c->st)
+             : copy_transpose(c->theta.p, mrow, ncol, false, c->jw.p, c->fp64, c->st));
+    c->stats.kernel_launches++;
+  }
+  TRY(svd_columns(c, rows, cols, c->sweep_cut, false, 0.0, k, f));
+  TRY(ensure(c, out, (size_t)rows * k * c->esz));
+  Span sp(c, TC_SVD);
+  CK(gather_columns(c->jw.p, rows, c->svd_n, k, c->tres.p, false, right ? 2 : 0, out.p, c->fp64, c->st));
+  c->stats.kernel_launches++;
+  return DMRGC_OK;
+}
+
 dmrgc_status update_ltr(dmrgc_ctx* c, int i) {
   // X_i from the running left environment
   EnvRef L = c->L;
@@ -754,7 +780,7 @@ dmrgc_status update_ltr(dmrgc_ctx* c, int i) {
   TRY(form_theta(c, i, mrow, ncol));
   std::vector<float> rec;
   TRY(record_begin(c, i, std::min(mrow, ncol), rec));
-  int k = 0, nnz = 0, l = 0;
+  int k = 0, l = 0;
   double f = 0;
   bool sketched = false;
   TRY(sketch_size(c, i, mrow, ncol, l));
@@ -763,21 +789,7 @@ dmrgc_status update_ltr(dmrgc_ctx* c, int i) {
   if (sketched) {
     TRY(record_end(c, i, k, false, rec));
   } else {
-    // U_k: leading eigenvectors of theta theta^+ where they are resolved, else Jacobi
-    TRY(eig_try(c, i, c->theta.p, mrow, ncol, false, c->sweep_cut, 0.0, c->A[i], 0, k, eig, true));
-    if (!eig) {
-      TRY(ensure(c, c->jw, (size_t)mrow * ncol * c->esz));
-      {
-        Span sp(c, TC_OTHER);
-        CK(copy_transpose(c->theta.p, mrow, ncol, false, c->jw.p, c->fp64, c->st));
-        c->stats.kernel_launches++;
-      }
-      TRY(svd_columns(c, mrow, ncol, c->sweep_cut, false, 0.0, k, f, &nnz));
-      TRY(ensure(c, c->A[i], (size_t)mrow * k * c->esz));
-      Span sp(c, TC_SVD);
-      CK(gather_columns(c->jw.p, mrow, c->svd_n, k, c->tres.p, false, 0, c->A[i].p, c->fp64, c->st));
-      c->stats.kernel_launches++;
-    }
+    TRY(svd_theta(c, i, false, mrow, ncol, c->A[i], k, f, eig));
     note_resolvable(c, i);
     TRY(record_end(c, i, k, true, rec));
   }
@@ -822,7 +834,7 @@ dmrgc_status update_rtl(dmrgc_ctx* c, int i) {
   TRY(form_theta(c, i, mrow, ncol));
   std::vector<float> rec;
   TRY(record_begin(c, i, std::min(mrow, ncol), rec));
-  int k = 0, nnz = 0, l = 0;
+  int k = 0, l = 0;
   double f = 0;
   bool sketched = false;
   TRY(sketch_size(c, i, mrow, ncol, l));
@@ -831,22 +843,7 @@ dmrgc_status update_rtl(dmrgc_ctx* c, int i) {
   if (sketched) {
     TRY(record_end(c, i, k, false, rec));
   } else {
-    // V_k^+: leading eigenvectors of theta^+ theta (conjugated rows) where resolved, else Jacobi
-    TRY(eig_try(c, i, c->theta.p, ncol, mrow, true, c->sweep_cut, 0.0, c->A[i + 1], 2, k, eig, true));
-    if (!eig) {
-      TRY(ensure(c, c->jw, (size_t)mrow * ncol * c->esz));
-      {
-        Span sp(c, TC_OTHER);
-        CK(copy_conj(c->theta.p, (long long)mrow * ncol, c->jw.p, c->fp64, c->st));
-        c->stats.kernel_launches++;
-      }
-      // columns of theta^+ (column-major == conj(theta) row-major): ncol rows, mrow columns
-      TRY(svd_columns(c, ncol, mrow, c->sweep_cut, false, 0.0, k, f, &nnz));
-      TRY(ensure(c, c->A[i + 1], (size_t)k * ncol * c->esz));
-      Span sp(c, TC_SVD);
-      CK(gather_columns(c->jw.p, ncol, c->svd_n, k, c->tres.p, false, 2, c->A[i + 1].p, c->fp64, c->st));
-      c->stats.kernel_launches++;
-    }
+    TRY(svd_theta(c, i, true, mrow, ncol, c->A[i + 1], k, f, eig));
     note_resolvable(c, i);
     TRY(record_end(c, i, k, true, rec));
   }
@@ -2244,6 +2241,51 @@ dmrgc_status dmrgc_test_svd(int precision, int m, int n, const double* G, int ch
   if (gather_columns(dG, m, n, tr.k, res, false, 0, dU, fp64, 0) != cudaSuccess) return DMRGC_ECUDA;
   if (download_from(dU, (long long)m * tr.k, fp64, s, U_out) != cudaSuccess) return DMRGC_ECUDA;
   return cudaDeviceSynchronize() == cudaSuccess ? DMRGC_OK : DMRGC_ECUDA;
+}
+
+dmrgc_status dmrgc_test_svd_theta(int precision, int svd_path, int right, int m, int n, const double* G, int chi,
+                                  double rel_cut, int* k_out, double* U_out, int* parts_out) {
+  if (precision < 0 || precision > 3 || svd_path < 0 || svd_path > 1 || right < 0 || right > 1 || m < 1 || n < 1 ||
+      m > 8192 || n > 8192 || chi < 1 || chi > 4096 || !(rel_cut > 0) || !G || !k_out || !U_out || !parts_out)
+    return DMRGC_EINVAL;
+  dmrgc_options o;
+  dmrgc_default_options(&o);
+  o.precision = precision;
+  o.svd_path = svd_path;
+  o.sweep_rel_cutoff = rel_cut;
+  const dmrgc_grid grid = {1, 2, 0};
+  dmrgc_ctx* c = nullptr;
+  dmrgc_status st = dmrgc_create(2, &grid, chi, &o, &c);
+  if (st != DMRGC_OK) return st;
+  st = [&]() -> dmrgc_status {
+    Scratch s;
+    void* dG;
+    if (upload_as(G, (long long)m * n, c->fp64, s, &dG) != cudaSuccess) return DMRGC_ECUDA;
+    // theta = G (right: G^+): row-major from the column-major G
+    TRY(ensure(c, c->theta, (size_t)m * n * c->esz));
+    CK(right ? copy_conj(dG, (long long)m * n, c->theta.p, c->fp64, c->st)
+             : copy_transpose(dG, n, m, false, c->theta.p, c->fp64, c->st));
+    int k = 0;
+    double f = 0;
+    bool eig = false;
+    TRY(svd_theta(c, 0, right != 0, right ? n : m, right ? m : n, c->A[0], k, f, eig));
+    const long long elems = (long long)m * k;
+    if (right) {   // U_k from U_k^+ [k][m]
+      void* u = s.get((size_t)elems * c->esz);
+      void* v = s.get((size_t)elems * c->esz);
+      if (!u || !v) return DMRGC_ENOMEM;
+      CK(copy_conj(c->A[0].p, elems, u, c->fp64, c->st));
+      CK(copy_transpose(u, k, m, false, v, c->fp64, c->st));
+      CK(download_from(v, elems, c->fp64, s, U_out));
+    } else {
+      CK(download_from(c->A[0].p, elems, c->fp64, s, U_out));
+    }
+    *k_out = k;
+    *parts_out = c->eig_parts;
+    return DMRGC_OK;
+  }();
+  dmrgc_destroy(c);
+  return st;
 }
 
 void dmrgc_destroy(dmrgc_ctx* c) {

@@ -52,6 +52,7 @@ struct dmrgc_ctx {
   DevBuf ework;    // work space of the Gram eigensolver path (eig_truncate)
   DevBuf df_r, df_c, df_u[4];   // its stages: the residual, U^+ residual, the vectors of each stage
   TruncResult last_tr{};          // result of the last truncated SVD (either path)
+  int eig_parts = 0;              // Gram matrices the last eigensolver SVD took its vectors from (0: it took none)
   int svd_n = 0;                  // columns of the matrix the last Jacobi SVD ended with (svd_columns)
   std::vector<char> eig_declined; // per bond: the eigensolver's most capable form that declined it in this layer (eig_try)
   DevBuf rv[3];    // read-outs: running rows V, site products W = V A_i, T = W E_i

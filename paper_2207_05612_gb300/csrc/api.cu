@@ -234,7 +234,7 @@ dmrgc_status svd_columns(dmrgc_ctx* c, int m, int n, double rel_cut, bool square
 // given as theta = G^+, kdim x rows) are the leading eigenvectors of H = G G^+,
 // formed by the contraction engine with TF32x3 split products (FP32 CUDA cores in
 // the FP32 mode).  done = false: the caller runs the Jacobi SVD.  out receives
-// the k vectors in layout `mode` (see eig_truncate).
+// the k vectors in layout `mode` (see eig_select).
 //
 // lambda_{k-1} >= 1e-5 lambda_0 (s_{k-1} >= 3e-3 s_1): ten times the Gram
 // path's absolute eigenvalue error (~1e-6 lambda_0 for a TF32x3 Gram and an
@@ -1014,10 +1014,13 @@ dmrgc_status zip_guess(dmrgc_ctx* c) {
 //  right to left:  W_i = L Q' with orthonormal rows Q',  W_{i-1} <- W_{i-1} L.
 // After the first pass the left part is an isometry, so the second pass sees
 // the true operator Schmidt values.  A cut at full rank is left as it is.
-// The LQ reduction pays from 65 columns on here.  Below, it would also replace the
-// sparse site tensors by dense ones before their SVD, whose bases the split
-// products round differently (BF16x3: partial fidelities moved by 1.2e-5 on
-// average, 5e-6 without).
+// The LQ reduction is used from 65 columns on here.  Below, it is faster too, but it
+// replaces the sparse site tensors by dense ones before their SVD, whose bases the
+// BF16x3 products round differently: partial fidelities move by 1e-5, further than
+// anything else here moves them, so the line keeps results where they were.  It is
+// not the more exact side (4 x 5, chi = 256, median of eight states, BF16x3 against FP64:
+// -6.4e-5 without LQ, -5.5e-5 with this line, -4.5e-5 with LQ at any width; 4 x 4, chi =
+// 200: -2.6e-5, -1.8e-5, -1.0e-5; TF32x3: the three agree to 2e-6).
 constexpr int kMpoLq = 65;
 
 dmrgc_status compress_mpo(dmrgc_ctx* c) {
@@ -2181,7 +2184,8 @@ dmrgc_status dmrgc_test_svd_gram(int precision, int m, int n, const double* G, i
   g.upper_only = 1;
   TcWork w;
   cudaError_t e = run_gemm(precision == DMRGC_FP32 ? DMRGC_FP32 : DMRGC_TF32X3, g, &w, err, 0);
-  if (e == cudaSuccess) e = eig_truncate(dH, m, chi, rel_cut, 0.0, kEigResolve, work, res, dU, 0, 0, nullptr);
+  if (e == cudaSuccess) e = eig_reduce(dH, m, kk, work, 0, nullptr);
+  if (e == cudaSuccess) e = eig_select(dH, m, kk, chi, rel_cut, 0.0, kEigResolve, work, res, dU, 0, 0, nullptr);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   w.release();
   if (e != cudaSuccess) return DMRGC_ECUDA;

@@ -153,7 +153,10 @@ cudaError_t gather_columns(const void* W, int m, int n_total, int k, const void*
                            bool squared, int mode, void* out, bool fp64, cudaStream_t st);
 
 // Truncated SVD through the Gram matrix's eigenproblem (eig_herm.cu), complex64.
-// H: n x n row-major Hermitian (overwritten), 3 <= n <= 2048.  Keeps
+// eig_reduce: H (n x n row-major Hermitian, 3 <= n <= 2048) <- its tridiagonal form
+// and reflectors, the kk leading eigenvalues by bisection.  eig_spectrum: those on
+// the host (in units of head->unit; synchronises st).  eig_select, any number of
+// times after one eig_reduce with the same n, kk and work: keeps
 // k = min(chi, n, #{s > cut s_1}) with the multiplet rule of tie_rel (> 0)
 // and writes res (TruncResult + s[n] + perm[n], as truncate_columns) and the
 // k leading eigenvectors to out: mode 0 out[r * k + v], mode 1 out[v * n + r],
@@ -162,13 +165,6 @@ cudaError_t gather_columns(const void* W, int m, int n_total, int k, const void*
 // cut^2 < resolve: use the Jacobi SVD; nothing is written to out);
 // DMRGC_ENUMERIC; DMRGC_ETIMEOUT.
 size_t eig_work_bytes(int n, int kk);
-cudaError_t eig_truncate(void* H, int n, int chi, double cut, double tie_rel, double resolve, void* work,
-                         void* res, void* out, int mode, cudaStream_t st, int* launches);
-// The same in two parts.  eig_reduce: H <- its tridiagonal form and reflectors,
-// the kk leading eigenvalues by bisection.  eig_spectrum: those on the host (in
-// units of head->unit; synchronises st).  eig_select: vectors, truncation and
-// back-transformation as eig_truncate, any number of times after one
-// eig_reduce with the same n, kk and work.
 struct EigHead {
   int err;         // 0 or DMRGC_ETIMEOUT
   double unit;     // eigenvalue of the H given to eig_reduce per unit of lam

@@ -49,7 +49,7 @@ struct dmrgc_ctx {
   DevBuf envL, envR, T, theta, jw, bt, one, jctl, tres, scal, gates_d, rank_d, fa_d, fb_d, plan_d;
   DevBuf ptrs_d, bonds_d, order_d, bits_d, out_d, stage_d, tcerr;
   DevBuf ovl[2];   // ping-pong environments of dmrgc_overlap (never the sweep's envL / envR)
-  DevBuf ework;    // work space of the Gram eigensolver path (eig_truncate)
+  DevBuf ework;    // work space of the Gram eigensolver path (eig_reduce, eig_select)
   DevBuf df_r, df_c, df_u[4];   // its stages: the residual, U^+ residual, the vectors of each stage
   TruncResult last_tr{};          // result of the last truncated SVD (either path)
   int eig_parts = 0;              // Gram matrices the last eigensolver SVD took its vectors from (0: it took none)

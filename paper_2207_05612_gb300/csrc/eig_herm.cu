@@ -51,13 +51,11 @@ namespace {
 struct HeCtl {
   int err;            // 0 ok, DMRGC_ETIMEOUT
   unsigned count;     // grid-barrier arrivals of the tridiagonalisation (never reset in a launch)
-  unsigned gen;       // (unused)
   int status;         // inverse iteration / clusters: 0 ok, 1 not resolved
   float scale;        // max(|d|, |beta|) of T, for the tridiagonal kernels
-  int pad0;
   double gscale;      // max_i H_ii: H was divided by it
   double trace;       // trace of the scaled H
-  int pad[6];
+  int pad[8];
 };
 static_assert(sizeof(HeCtl) == 64, "control block layout");
 
@@ -1367,7 +1365,7 @@ __global__ void __launch_bounds__(BT_WARPS * 32)
   }
 }
 
-// work-space layout of eig_truncate, parts rounded to 256 bytes
+// work-space layout of eig_reduce and eig_select, parts rounded to 256 bytes
 constexpr int kParts = 13;
 
 struct EigParts {
@@ -1582,15 +1580,6 @@ cudaError_t eig_select(const void* H, int n, int kk, int chi, double cut, double
   }
   if (launches) *launches += 5;
   return cudaSuccess;
-}
-
-cudaError_t eig_truncate(void* H, int n, int chi, double cut, double tie_rel, double resolve, void* work,
-                         void* res, void* out, int mode, cudaStream_t st, int* launches) {
-  if (n < 3 || n > 2048 || chi < 1) return cudaErrorInvalidValue;
-  const int kk = chi + 1 < n ? chi + 1 : n;
-  const cudaError_t e = eig_reduce(H, n, kk, work, st, launches);
-  if (e != cudaSuccess) return e;
-  return eig_select(H, n, kk, chi, cut, tie_rel, resolve, work, res, out, mode, st, launches);
 }
 
 }  // namespace dmrgc

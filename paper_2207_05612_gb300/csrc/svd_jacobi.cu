@@ -1450,8 +1450,16 @@ bool try_cluster_jacobi(void* G, int m, int n, double tol, double conv, int max_
                         double zero_rel, JacobiCtl* c, cudaStream_t st, cudaError_t& err) {
   using C2 = typename cplx<R>::T;
   const void* fn;
-  int E, wmax;   // rows of a column per lane, most columns per block (128 KB of shared memory)
+  int E, w, wmax;   // rows of a column per lane; columns per block, at most (128 KB of shared memory)
+  // complex64 is bound by the latency of a sub-round: w = 4 up to 128 columns
+  // (64 x 64: 0.37 ms; w = 2: 0.52 ms, more hops between SMs; 128 x 100: 0.65
+  // ms, w = 8: 0.90 ms before the shorter rotation), w = 8 up to 256.
+  // FP64: a warp's FP64 instruction holds a quarter of its SM for 64 cycles, so
+  // the work has to spread over many SMs: w = 2 (64 x 64: 1.84 ms; w = 4: 2.77 ms,
+  // w = 8: about 5 ms), and beyond 64 columns, where a cluster would need wider
+  // blocks, the grid-wide kernel takes over (200 x 96: 6.5 ms, cluster 8.9 ms).
   if constexpr (sizeof(R) == 4) {
+    w = 4;
     const bool vec = m % 2 == 0 && (reinterpret_cast<uintptr_t>(G) % 16) == 0;
     if (m <= 64) { E = 2; wmax = 8; fn = jc_fn<R, 2, 512>(vec); }
     else if (m <= 128) { E = 4; wmax = 8; fn = jc_fn<R, 4, 512>(vec); }
@@ -1459,22 +1467,15 @@ bool try_cluster_jacobi(void* G, int m, int n, double tol, double conv, int max_
     else if (m <= 512) { E = 16; wmax = 4; fn = jc_fn<R, 16, 256>(vec); }
     else return false;
   } else {
-    if (m <= 32) { E = 1; wmax = 8; fn = jc_fn<R, 1, 512>(false); }
-    else if (m <= 64) { E = 2; wmax = 8; fn = jc_fn<R, 2, 512>(false); }
-    else if (m <= 128) { E = 4; wmax = 8; fn = jc_fn<R, 4, 512>(false); }
-    else if (m <= 256) { E = 8; wmax = 4; fn = jc_fn<R, 8, 256>(false); }
-    else if (m <= 512) { E = 16; wmax = 2; fn = jc_fn<R, 16, 128>(false); }
+    if (n > 64) return false;
+    w = wmax = 2;
+    if (m <= 32) { E = 1; fn = jc_fn<R, 1, 128>(false); }
+    else if (m <= 64) { E = 2; fn = jc_fn<R, 2, 128>(false); }
+    else if (m <= 128) { E = 4; fn = jc_fn<R, 4, 128>(false); }
+    else if (m <= 256) { E = 8; fn = jc_fn<R, 8, 128>(false); }
+    else if (m <= 512) { E = 16; fn = jc_fn<R, 16, 128>(false); }
     else return false;
   }
-  // FP64: a warp's FP64 instruction holds a quarter of its SM for 64 cycles, so
-  // the work has to spread over many SMs: w = 2 (64 x 64: 1.84 ms; w = 4: 2.77 ms,
-  // w = 8: about 5 ms), and beyond 64 columns, where a cluster would need wider
-  // blocks, the grid-wide kernel takes over (200 x 96: 6.5 ms, cluster 8.9 ms).
-  // complex64 is bound by the latency of a sub-round: w = 4 up to 128 columns
-  // (64 x 64: 0.37 ms; w = 2: 0.52 ms, more hops between SMs; 128 x 100: 0.65
-  // ms, w = 8: 0.90 ms before the shorter rotation), w = 8 up to 256.
-  if (sizeof(R) == 8 && n > 64) return false;
-  int w = sizeof(R) == 8 ? 2 : 4;
   while (w < wmax && (n + 2 * w - 1) / (2 * w) > 16) w *= 2;
   const int ctas = (n + 2 * w - 1) / (2 * w);
   if (ctas > 16) return false;

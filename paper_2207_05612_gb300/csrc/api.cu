@@ -270,14 +270,17 @@ bool eig_applies(const dmrgc_ctx* c, int rows, int kdim, bool sweep) {
 }
 
 // The form it takes a matrix in, by what it resolves.  0: it does not take it;
-// 1: one Gram matrix; 2: one, and the residual if that is noise; 3: stages.
+// 1: one Gram matrix; 2: one, and the residual if that is noise; 3: stages.  One Gram
+// matrix of rank below chi never resolves the sweep's cut: the rank is then set by it.
 // Stages run where the spectrum itself is not recorded, above 256 rows, and below that,
 // as form 2, where rows need not be dropped: the usual case there is a matrix of
 // lower rank, which ends with the first residual (a second diagonalisation
 // would be slower than the cluster Jacobi kernel: eig_try declines).
 int eig_form(const dmrgc_ctx* c, int rows, int kdim, bool sweep) {
   if (!eig_applies(c, rows, kdim, sweep)) return 0;
-  if (!sweep || (rows <= 256 && c->chi < rows) || c->opt.svd_mode != 0 || c->opt.log_rank_records) return 1;
+  if (!sweep) return 1;
+  if ((rows <= 256 && c->chi < rows) || c->opt.svd_mode != 0 || c->opt.log_rank_records)
+    return kdim < std::min(rows, c->chi) && c->sweep_cut * c->sweep_cut < kEigResolve ? 0 : 1;
   return rows > 256 ? 3 : 2;
 }
 

@@ -144,6 +144,12 @@ static void visits() {
   g_status = 0;
   update(e, "stages", 400, 400, true);
   update(e, "stages", 250, 400, false);
+  dmrgc_ctx l;
+  setup(l, 200, 4);   // rank below chi: the sweep's cut sets the count, a wider one is resolved
+  update(l, "low rank", 250, 150, false);
+  update(l, "low rank", 250, 200, false);
+  l.sweep_cut = 4e-3;
+  update(l, "low rank, wide cut", 250, 150, false);
   dmrgc_ctx r;
   setup(r, 200, 4);
   r.opt.log_rank_records = 1;   // the recorded spectrum decides

@@ -65,6 +65,9 @@ def test_bond_visits(host):
         "stages 400 x 400 left to right: declined",
         "stages 400 x 400 right to left: skipped",
         "stages 250 x 400 left to right: skipped",
+        "low rank 250 x 150 left to right: not tried",
+        "low rank 250 x 200 left to right: taken",
+        "low rank, wide cut 250 x 150 left to right: taken",
         "records 400 x 400 left to right: declined",
         "records 400 x 400 right to left: taken",
     ]

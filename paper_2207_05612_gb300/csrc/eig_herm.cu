@@ -452,6 +452,13 @@ __global__ void __launch_bounds__(TD_THREADS, 1)
 // become one hop between SMs (1.7 us at 256 rows; 2.25 us at 512, where the rank-2
 // update of 32 rows per SM takes 0.85).  Of a step at 256 rows, 3700 cycles, the
 // rows take 980, the exchange 900, the two reductions 870, the reflector 480.
+// An entry takes its four products one by one, four roundings a step where the
+// grid-wide kernel has one: of a spectrum without gaps the span of the kept half
+// misses 4.0e-13 of the weight at 256 rows (grid-wide 2.5e-13) and 6.7e-13 at 512
+// (3.9e-13).  Summing the update first brings 2.2e-13 and 3.2e-13 for 1 to 4% of the
+// time, but moves states whose cuts fall into near-degenerate multiplets by more than
+// the rounding it saves (one run in four of those drawn at odd chi, by 1e-3 to 1e-2
+// in single f), as any change of rounding does.
 // One cluster leaves the other SMs to other streams.  (Eight clusters holding
 // 1024 rows that passed packets through L2 gained 3% over the grid-wide kernel:
 // left out.)

@@ -145,8 +145,8 @@ typedef struct {
   long long eig_svds;           /* truncated SVDs done by the Gram eigensolver (svd_path 0) */
   long long eig_fallbacks;      /* Gram eigensolver results not resolved or not finite: redone by
                                    Jacobi */
-  long long eig_skipped;        /* SVDs sent straight to Jacobi: the last one at that bond was not
-                                   resolvable by the eigensolver */
+  long long eig_skipped;        /* SVDs sent straight to Jacobi: in this layer the eigensolver had
+                                   declined one at that bond in a form that resolves as much */
 } dmrgc_stats;
 
 /* Fill *opt with defaults (FP64, Jacobi, default cutoffs, default stream). */

@@ -111,7 +111,7 @@ int gemm_tc_split(int M, int N, int K, int precision);
 // In complex64 such a column is left as it is even when it holds part of a value above
 // the level, so that of a spectrum that decays through it the rank comes out short and
 // the last values low (300 x 512, five decades: 239 of 267 values above it kept, 1e-8
-// of the weight missed; with a quarter of the level 264 and 3e-10, and 15% more time).
+// of the weight missed; with a quarter of the level 264 and 3e-10, and 20% more time).
 // n_out (optional): a wide matrix (m < n) may be replaced by the L of its LQ
 // factorisation, which has the same left singular vectors and values; *n_out
 // receives the columns that G then has (m, else n).

@@ -449,9 +449,10 @@ __global__ void __launch_bounds__(TD_THREADS, 1)
 // goes to a CTA that has left.
 // Bound by the latency of that chain: a grid-wide atomic barrier and two L2
 // round trips per column (5.9 us at 1024 rows, about 4.4 us at 256 to 512)
-// become one hop between SMs (1.7 us at 256 rows; 2.25 us at 512, where the rank-2
-// update of 32 rows per SM takes 0.85).  Of a step at 256 rows, 3700 cycles, the
-// rows take 980, the exchange 900, the two reductions 870, the reflector 480.
+// become one hop between SMs (1.6 us at 256 rows; 2.1 us at 512, where the rank-2
+// update of 32 rows per SM takes 0.85).  Of a step at 256 rows, 3700 cycles before the
+// vectors were loaded a block ahead, the rows took 980, the exchange 900, the two
+// reductions 870, the reflector 480.
 // An entry takes its four products one by one, four roundings a step where the
 // grid-wide kernel has one: of a spectrum without gaps the span of the kept half
 // misses 4.0e-13 of the weight at 256 rows (grid-wide 2.5e-13) and 6.7e-13 at 512

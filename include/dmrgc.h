@@ -102,7 +102,9 @@ typedef struct {
                                  straddling gates' Schmidt ranks */
   int svd_path;               /* complex64 modes, truncated SVDs of 128..2048 rows that keep
                                  fewer than all of them (the sweep's theta, the zip-up's Gram)
-                                 and, in the sweep, of more than 192 rows that may keep all:
+                                 and, in the sweep, of more than 192 rows that may keep all
+                                 (not tall thetas of few columns, nor those of at most 256
+                                 rows whose rank is below chi < rows):
                                  0 (default) = the leading eigenvectors of the Gram matrix
                                  G G^+ (TF32x3 product, Householder tridiagonalisation,
                                  bisection and FP64 inverse iteration, back-transformation)
